@@ -219,7 +219,17 @@ def kernel_bytes_per_voxel(D=3, fp=4):
             "rows_inv": C * cb * 3 + medium,   # w, x in; x out
             "plane_fwd": C * cb * 3 + medium,  # x-y plane kernels: the same reads and writes as the row kernels
             "plane_inv": C * cb * 3 + medium,
-            "rows_inv_fwd": C * cb * 5 + medium}  # w, x, y in; x, w out (update + next forward transform)
+            "rows_inv_fwd": C * cb * 5 + medium,  # w, x, y in; x, w out (update + next forward transform)
+            **_scalar_form_bytes(D, fp, medium)}
+
+
+def _scalar_form_bytes(D, fp, medium):
+    """The kernels of the iteration that carries one scalar sum in place of the merged components: the y axis takes
+    three fields to two and back, the last axis two to two, and the row kernel reads x, y, the medium and D fields of
+    w and writes x and D fields of w."""
+    C, cb = D + 1, 2 * fp
+    return {"axis_merge": cb * 5, "last_solve": cb * 4, "axis_split": cb * 5,
+            "rows_update": (3 * C + 2 * D) * cb + medium}
 
 
 def model_bytes_per_voxel(D=3, fp=4):
@@ -232,7 +242,8 @@ def model_bytes_per_voxel(D=3, fp=4):
     medium = 3 * fp
     return {"rows_fwd": C * cb * 3 + medium, "axis_fwd": C * cb * 2, "last_symbol": C * cb * 2,
             "axis_inv": C * cb * 2, "rows_inv": C * cb * 3 + medium, "plane_fwd": C * cb * 3 + medium,
-            "plane_inv": C * cb * 3 + medium, "rows_inv_fwd": C * cb * 5 + medium}
+            "plane_inv": C * cb * 3 + medium, "rows_inv_fwd": C * cb * 5 + medium,
+            **_scalar_form_bytes(D, fp, medium)}
 
 
 def run_gpu(args):
@@ -302,11 +313,11 @@ def run_gpu(args):
         e1.record(stream)
         torch.cuda.synchronize()
         t64 = e0.elapsed_time(e1)
-        # the float64 path is bound by the FP64 pipes: its flop rate (5 log2(N_v) flops per point per transform,
-        # forward and inverse, C components, plus ~100 for the symbol and the pointwise steps) against the
-        # measured FP64 FMA rate of this GPU
+        # the float64 path is bound by the FP64 pipes: its flop rate (5 log2(n) flops per point per 1-D transform, 18
+        # of them an iteration: 8 along x, 6 along y, 4 along z, plus ~200 for the factors, the solve and the
+        # update) against the measured FP64 FMA rate of this GPU
         fp64_peak = cbs.fp64_rate()
-        flops_per_vi = 2 * 4 * 5 * np.log2(Nv) + 100
+        flops_per_vi = 18 * 5 * np.log2(p.shape[0]) + 200
         fp64_tflops = flops_per_vi * Nv * i64["iters"] / (t64 / 1e3) / 1e12
         fp64 = {"time_to_1e-6_ms": t64, "iters": i64["iters"], "rel_residual": i64["rel_residual"],
                 "voxel_iters_per_s": Nv * i64["iters"] / (t64 / 1e3),

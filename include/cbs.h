@@ -214,7 +214,7 @@ cbs_status solver_time_kernels(cbs_solver* s, const void* y, void* x, int n_iter
  * caller-owned device complex128 [C][N] buffers; out is also the work array.
  * Work is enqueued on `stream` (cudaStream_t, may be 0) and the call
  * synchronises that stream before it returns.  It allocates no device memory:
- * its tables and norm partials live in a static device array of 124 KiB that
+ * its tables live in a static device array of 84 KiB that
  * every GPU loading the library holds until exit.  The first call on each
  * device looks up that array's device address (cudaGetSymbolAddress) and keeps
  * it for the life of the process, so make the first call on a device before

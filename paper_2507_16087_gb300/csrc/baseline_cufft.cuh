@@ -33,29 +33,39 @@ __global__ void k_base_pre(Dims d, Medium<R> M, const cplx<R>* __restrict__ x, c
     }
 }
 
-// the per-wavenumber symbol on the C components of each k (the 1/N of the
-// unnormalised inverse transform is in the symbol constants)
-template <typename R, int C>
-__global__ void k_base_symbol(Dims d, Symbol<R> Sy, cplx<R>* __restrict__ w, int mode)
+// constants of the per-wavenumber (L+I)^-1 (App. B.1, forward or conjugated for the adjoint)
+struct BaseSymbol {
+    float2 P, Pu, c1, c2, c3;  // l1/(a1+l1)/N, l1/(a1+l1), i sqrt(l1 l2), l2 (a1+l1), (a1+l1)(a2+l2)
+    float scale;               // 1/N
+    const float2* kt[3];       // t_eta
+    const float* k2[3];
+};
+
+// the per-wavenumber symbol on the C components of each k
+template <int C> __global__ void k_base_symbol(Dims d, BaseSymbol Sy, float2* __restrict__ w)
 {
     constexpr int D = C - 1;
     for (long long v = blockIdx.x * (long long)blockDim.x + threadIdx.x; v < d.N; v += (long long)gridDim.x * blockDim.x) {
         int i0, i1, i2;
         voxel_coords(d, v, i0, i1, i2);
-        cplx<R> t[D];
-        t[0] = Sy.kt[0][i0];
-        t[1] = Sy.kt[1][i1];
-        R k2 = Sy.k2[0][i0] + Sy.k2[1][i1];
-        if constexpr (D == 3) {
-            t[2] = Sy.kt[2][i2];
-            k2 += Sy.k2[2][i2];
-        }
-        cplx<R> vv[C];
+        const int ix[3] = {i0, i1, i2};
+        float2 vv[C], t[D], s = make_float2(0.f, 0.f);
+        float k2 = 0.f;
 #pragma unroll
         for (int c = 0; c < C; ++c) vv[c] = w[c * d.N + v];
-        apply_symbol<R, C>(Sy, mode, t, k2, vv);
 #pragma unroll
-        for (int c = 0; c < C; ++c) w[c * d.N + v] = vv[c];
+        for (int e = 0; e < D; ++e) {
+            t[e] = Sy.kt[e][ix[e]];
+            k2 += Sy.k2[e][ix[e]];
+            s = cadd(s, cmulc(vv[e], t[e]));
+        }
+        const float2 mu = make_float2(k2 + Sy.c3.x, Sy.c3.y);
+        const float inv = Sy.scale / cabs2(mu);
+        const float2 im = make_float2(mu.x * inv, -mu.y * inv);
+        const float2 tmp = cmul(cadd(cmul(Sy.Pu, s), cmul(Sy.c1, vv[D])), im);
+#pragma unroll
+        for (int e = 0; e < D; ++e) w[e * d.N + v] = csub(cmul(Sy.P, vv[e]), cmul(t[e], tmp));
+        w[D * d.N + v] = cmul(csub(cmul(Sy.c2, vv[D]), cmul(Sy.c1, s)), im);
     }
 }
 

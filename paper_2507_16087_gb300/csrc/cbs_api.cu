@@ -3,20 +3,20 @@
 // operator entry points used for step-by-step checks.  All compute runs in
 // the kernels of born.cuh and the set-up/utility kernels below; the host
 // only computes O(n) per-axis tables and scalars.
-#include <cuda.h>
-#include <cudaTypedefs.h>
 #include <cuda_runtime.h>
 #include <cufft.h>
 
 #include <algorithm>
 #include <type_traits>
 #include <cmath>
+#include <complex>
 #include <cstdint>
 #include <cstdio>
 #include <cstdlib>
 #include <cstring>
 #include <string>
 #include <mutex>
+#include <utility>
 #include <vector>
 
 #include "cbs.h"
@@ -469,6 +469,10 @@ struct cbs_solver {
     double* k264[3] = {};
     float2* kt32[3] = {};
     float* k232[3] = {};
+    std::vector<double2> kt_host[3];
+    // merge / split factors of (L+I)^-1 per axis, [adjoint][axis]
+    double2 *tm64[2][3] = {}, *td64[2][3] = {};
+    float2 *tm32[2][3] = {}, *td32[2][3] = {};
     double2* tw64[3] = {};
     float2* tw32[3] = {};
 
@@ -486,6 +490,7 @@ struct cbs_solver {
     cudaGraphExec_t graph64[2] = {nullptr, nullptr};
     cudaGraphExec_t graph32[2] = {nullptr, nullptr};
     bool warmed64 = false, warmed32 = false;
+    long long graph_launches[2] = {};  // kernels in one replay of a float64 / float32 block
     int hist_n = 0;          // entries of hist written by the last block
     int* errword = nullptr;  // device error word of the bulk-staged kernels
     cudaAccessPolicyWindow l2_window{};
@@ -580,10 +585,26 @@ double layer_gamma(double xi, long n, int lo, int hi, double gmax, double power)
     return d > 0.0 ? gmax * std::pow(d, power) : 0.0;
 }
 
-template <typename T> void upload(cbs_solver* s, T* dst, const std::vector<T>& v)
-{
-    CUDA_TRY(cudaMemcpyAsync(dst, v.data(), v.size() * sizeof(T), cudaMemcpyHostToDevice, s->st));
-}
+// Host-made tables gathered into one buffer, so that a set of them takes one allocation and one copy: add() hands out
+// a place (aligned to 256 bytes) and upload() sets every handed-out device pointer.  The buffer must live until the
+// stream has been synchronised.
+struct TablePack {
+    std::vector<unsigned char> bytes;
+    std::vector<std::pair<void**, size_t>> places;
+    template <typename T> void add(T** dst, const std::vector<T>& v)
+    {
+        const size_t at = (bytes.size() + 255) / 256 * 256;
+        bytes.resize(at + v.size() * sizeof(T));
+        std::memcpy(bytes.data() + at, v.data(), v.size() * sizeof(T));
+        places.emplace_back(reinterpret_cast<void**>(dst), at);
+    }
+    void upload(cbs_solver* s)
+    {
+        unsigned char* base = dalloc<unsigned char>(s, bytes.size());
+        for (auto& p : places) *p.first = base + p.second;
+        CUDA_TRY(cudaMemcpyAsync(base, bytes.data(), bytes.size(), cudaMemcpyHostToDevice, s->st));
+    }
+};
 
 // ---------------------------------------------------------------- iteration pieces
 template <typename R> struct Bufs;
@@ -594,6 +615,7 @@ template <> struct Bufs<double> {
     static double2* w(cbs_solver* s) { return s->w64; }
     static cudaGraphExec_t* graph(cbs_solver* s) { return s->graph64; }
     static bool& warmed(cbs_solver* s) { return s->warmed64; }
+    static long long& graph_launches(cbs_solver* s) { return s->graph_launches[0]; }
 };
 template <> struct Bufs<float> {
     static Plan<float>& plan(cbs_solver* s) { return s->P32; }
@@ -602,71 +624,41 @@ template <> struct Bufs<float> {
     static float2* w(cbs_solver* s) { return s->w32; }
     static cudaGraphExec_t* graph(cbs_solver* s) { return s->graph32; }
     static bool& warmed(cbs_solver* s) { return s->warmed32; }
+    static long long& graph_launches(cbs_solver* s) { return s->graph_launches[1]; }
 };
 
-// sum the partials of `nslots` slots into out[2 * slot]
-void reduce_slots(cbs_solver* s, int nblk, int nslots, double* out)
+// sum the partials of `nslots` slots (nblk pairs each) into out[2 * slot]
+void reduce_slots(cbs_solver* s, const double* part, int nblk, int nslots, double* out)
 {
-    k_reduce<<<nslots, 256, 0, s->st>>>(s->partials, nblk, out);
+    k_reduce<<<nslots, 256, 0, s->st>>>(part, nblk, out);
     CUDA_TRY(cudaGetLastError());
     s->launches += 1;
 }
 
-// one Born iteration on the precision-R buffers (eq. BornAlt); its norm
-// partials go to slot `slot`
-template <typename R> int iter_blocks(const Plan<R>& P) { return P.plane ? plane_blocks<R>(P) : rows_blocks<R>(P); }
-template <typename R> int iter_kernels(const Plan<R>& P) { return P.plane ? 3 : (P.d.D == 3 ? 5 : 3); }
-
-template <typename R> void iterate_once(cbs_solver* s, bool adj, int slot)
+// n <= kslots iterations (eq. BornAlt) on the precision-R buffers: the forward row kernel once, then per iteration
+// the strided-axis kernels and the row kernel that updates x and starts the next iteration; the last iteration ends
+// with the plain update.  norms: the increment of every iteration goes to hist[0..n), else only the last one's (a
+// solve reads no other).
+template <typename R> void iterate_block(cbs_solver* s, int n, bool adj, bool norms)
 {
     Plan<R>& P = Bufs<R>::plan(s);
     auto x = Bufs<R>::x(s);
     auto y = Bufs<R>::y(s);
     auto w = Bufs<R>::w(s);
-    const int nblk = iter_blocks<R>(P);
-    if (P.plane) {  // x-y plane kernels around the last-axis symbol kernel
-        CUDA_TRY(launch_plane_fwd<R>(P, x, y, w, adj, s->st));
-        CUDA_TRY(launch_last<R>(P, w, adj ? SYM_GREEN_ADJ : SYM_GREEN, s->st));
-        CUDA_TRY(launch_plane_inv<R>(P, x, w, adj, (R)s->opt.nu, s->partials + (size_t)slot * nblk * 2, s->st));
-        s->launches += 3;
-        return;
+    const int nblk = rows_blocks<R>(P);
+    const R nu = (R)s->opt.nu;
+    CUDA_TRY(launch_rows<R>(P, x, y, w, ROWS_FWD, adj, nu, nullptr, s->st));
+    s->launches += 1;
+    for (int k = 0; k < n; ++k) {
+        if (s->D == 3) CUDA_TRY(launch_axis<R>(P, w, -1, adj, s->st));
+        CUDA_TRY(launch_last<R>(P, w, adj, s->st));
+        if (s->D == 3) CUDA_TRY(launch_axis<R>(P, w, +1, adj, s->st));
+        const int mode = k + 1 == n ? ROWS_INV : (norms ? ROWS_FUSED_NORM : ROWS_FUSED);
+        CUDA_TRY(launch_rows<R>(P, x, y, w, mode, adj, nu, s->partials + (size_t)k * nblk * 2, s->st));
+        s->launches += (s->D == 3) ? 4 : 2;
     }
-    CUDA_TRY(launch_rows_fwd<R>(P, x, y, w, FWD_BORN, adj, s->st));
-    if (s->D == 3) CUDA_TRY(launch_axis<R>(P, w, -1, s->st));
-    CUDA_TRY(launch_last<R>(P, w, adj ? SYM_GREEN_ADJ : SYM_GREEN, s->st));
-    if (s->D == 3) CUDA_TRY(launch_axis<R>(P, w, +1, s->st));
-    CUDA_TRY(launch_rows_inv<R>(P, x, y, w, INV_BORN, adj, (R)s->opt.nu, s->partials + (size_t)slot * nblk * 2, s->st));
-    s->launches += (s->D == 3) ? 5 : 3;
-}
-
-// n <= kslots iterations and one reduction of their norms into hist[0..n).  With fused rows the update of
-// iteration k and the forward row transform of iteration k+1 are one kernel: the block launches the forward
-// row kernel once, then per iteration the strided-axis / last-axis kernels and the fused row kernel, the last
-// iteration ending with the plain update kernel.
-template <typename R> void iterate_block(cbs_solver* s, int n, bool adj)
-{
-    Plan<R>& P = Bufs<R>::plan(s);
-    if (P.plane || !P.fused_rows) {
-        for (int k = 0; k < n; ++k) iterate_once<R>(s, adj, k);
-    } else {
-        auto x = Bufs<R>::x(s);
-        auto y = Bufs<R>::y(s);
-        auto w = Bufs<R>::w(s);
-        const int nblk = rows_blocks<R>(P);
-        const R nu = (R)s->opt.nu;
-        CUDA_TRY(launch_rows_fwd<R>(P, x, y, w, FWD_BORN, adj, s->st));
-        s->launches += 1;
-        for (int k = 0; k < n; ++k) {
-            if (s->D == 3) CUDA_TRY(launch_axis<R>(P, w, -1, s->st));
-            CUDA_TRY(launch_last<R>(P, w, adj ? SYM_GREEN_ADJ : SYM_GREEN, s->st));
-            if (s->D == 3) CUDA_TRY(launch_axis<R>(P, w, +1, s->st));
-            double* part = s->partials + (size_t)k * nblk * 2;
-            if (k + 1 < n) CUDA_TRY(launch_rows_inv_fwd<R>(P, x, y, w, adj, nu, part, s->st));
-            else CUDA_TRY(launch_rows_inv<R>(P, x, y, w, INV_BORN, adj, nu, part, s->st));
-            s->launches += (s->D == 3) ? 4 : 2;
-        }
-    }
-    reduce_slots(s, iter_blocks<R>(P), n, s->hist);
+    if (norms) reduce_slots(s, s->partials, nblk, n, s->hist);
+    else reduce_slots(s, s->partials + (size_t)(n - 1) * nblk * 2, nblk, 1, s->hist + 2 * (n - 1));
 }
 
 // run n iterations in blocks of K = kslots; full blocks replay a captured CUDA graph
@@ -677,7 +669,7 @@ template <typename R> void run_iterations(cbs_solver* s, int n, bool adj)
     while (n > 0) {
         const int blk = std::min(n, K);
         if (!warmed || blk < K) {
-            iterate_block<R>(s, blk, adj);
+            iterate_block<R>(s, blk, adj, false);
             warmed = true;
         } else {
             cudaGraphExec_t& ge = Bufs<R>::graph(s)[adj ? 1 : 0];
@@ -686,12 +678,13 @@ template <typename R> void run_iterations(cbs_solver* s, int n, bool adj)
                 const long long l0 = s->launches;
                 CUDA_TRY(cudaStreamBeginCapture(s->st, cudaStreamCaptureModeThreadLocal));
                 try {
-                    iterate_block<R>(s, K, adj);
+                    iterate_block<R>(s, K, adj, false);
                 } catch (...) {
                     cudaStreamEndCapture(s->st, &g);
                     if (g) cudaGraphDestroy(g);
                     throw;
                 }
+                Bufs<R>::graph_launches(s) = s->launches - l0;
                 s->launches = l0;
                 CUDA_TRY(cudaStreamEndCapture(s->st, &g));
                 if (s->l2_window_set) {
@@ -713,42 +706,27 @@ template <typename R> void run_iterations(cbs_solver* s, int n, bool adj)
                 CUDA_TRY(e);
             }
             CUDA_TRY(cudaGraphLaunch(ge, s->st));
-            s->launches += (long long)K * iter_kernels<R>(Bufs<R>::plan(s)) + 1;
+            s->launches += Bufs<R>::graph_launches(s);
         }
         s->hist_n = blk;
         n -= blk;
     }
 }
 
-// w <- y - A_s x (mode INV_RESID) or w <- A_s x (INV_APPLY); red = (|w|^2, |y|^2)
-template <typename R> void apply_operator(cbs_solver* s, bool adj, int mode)
+// w <- y - A_s x; red = (|w|^2, |y|^2)
+template <typename R> void apply_residual(cbs_solver* s, bool adj)
 {
     Plan<R>& P = Bufs<R>::plan(s);
-    auto x = Bufs<R>::x(s);
-    auto y = Bufs<R>::y(s);
-    auto w = Bufs<R>::w(s);
-    CUDA_TRY(launch_rows_fwd<R>(P, x, y, w, FWD_COPY, adj, s->st));
-    if (s->D == 3) CUDA_TRY(launch_axis<R>(P, w, -1, s->st));
-    CUDA_TRY(launch_last<R>(P, w, adj ? SYM_L_ADJ : SYM_L, s->st));
-    if (s->D == 3) CUDA_TRY(launch_axis<R>(P, w, +1, s->st));
-    CUDA_TRY(launch_rows_inv<R>(P, x, y, w, mode, adj, (R)0, s->partials, s->st));
-    s->launches += (s->D == 3) ? 5 : 3;
-    reduce_slots(s, rows_blocks<R>(P), 1, s->red);
+    CUDA_TRY(launch_operator<R>(P, Bufs<R>::x(s), Bufs<R>::y(s), Bufs<R>::w(s), OP_RESID, adj, s->partials, s->st));
+    s->launches += s->D;
+    reduce_slots(s, s->partials, rows_blocks<R>(P), 1, s->red);
 }
 
-// w <- (L+I)^-1 x (or its adjoint)
-template <typename R> void apply_green(cbs_solver* s, bool adj)
+// whether two device ranges of n bytes share memory
+bool overlap(const void* a, const void* b, size_t n)
 {
-    Plan<R>& P = Bufs<R>::plan(s);
-    auto x = Bufs<R>::x(s);
-    auto y = Bufs<R>::y(s);
-    auto w = Bufs<R>::w(s);
-    CUDA_TRY(launch_rows_fwd<R>(P, x, y, w, FWD_COPY, adj, s->st));
-    if (s->D == 3) CUDA_TRY(launch_axis<R>(P, w, -1, s->st));
-    CUDA_TRY(launch_last<R>(P, w, adj ? SYM_GREEN_ADJ : SYM_GREEN, s->st));
-    if (s->D == 3) CUDA_TRY(launch_axis<R>(P, w, +1, s->st));
-    CUDA_TRY(launch_rows_inv<R>(P, x, y, w, INV_PLAIN, adj, (R)0, s->partials, s->st));
-    s->launches += (s->D == 3) ? 5 : 3;
+    const uintptr_t p = reinterpret_cast<uintptr_t>(a), q = reinterpret_cast<uintptr_t>(b);
+    return p < q + n && q < p + n;
 }
 
 void read_red(cbs_solver* s, double* out2)
@@ -774,7 +752,7 @@ void norm2_64(cbs_solver* s, const double2* a, long long n, double* out)
     k_norm2<<<g, 256, 0, s->st>>>(a, n, s->partials);
     CUDA_TRY(cudaGetLastError());
     s->launches += 1;
-    reduce_slots(s, g, 1, s->red);
+    reduce_slots(s, s->partials, g, 1, s->red);
     double r[2];
     read_red(s, r);
     *out = r[0];
@@ -873,7 +851,7 @@ template <typename R> cbs_status solve_plain(cbs_solver* s, bool adj, cbs_info* 
         inc = read_last_increment(s);
         if (tol > 0 && finite(inc) && gate.skip(inc, tol) && it < maxit) continue;
         if (tol > 0) {
-            apply_operator<R>(s, adj, INV_RESID);
+            apply_residual<R>(s, adj);
             double r[2];
             read_red(s, r);
             info->residual_checks++;
@@ -919,7 +897,7 @@ cbs_status solve_refine(cbs_solver* s, bool adj, cbs_info* info, bool zero_start
     if (zero_start) {
         CUDA_TRY(cudaMemcpyAsync(s->w64, s->y64, n * sizeof(double2), cudaMemcpyDeviceToDevice, s->st));
     } else {
-        apply_operator<double>(s, adj, INV_RESID);
+        apply_residual<double>(s, adj);
         read_red(s, r);
         info->residual_checks++;
         rn2 = r[0];
@@ -943,7 +921,7 @@ cbs_status solve_refine(cbs_solver* s, bool adj, cbs_info* info, bool zero_start
             inc = read_last_increment(s);
             if (!finite(inc)) { st = CBS_EDIVERGED; break; }
             if (gate.skip(inc, target) && it < maxit) continue;
-            apply_operator<float>(s, adj, INV_RESID);  // inner residual (float32)
+            apply_residual<float>(s, adj);  // inner residual (float32)
             double ri[2];
             read_red(s, ri);
             const double rr = std::sqrt(ri[0] / ri[1]);
@@ -956,7 +934,7 @@ cbs_status solve_refine(cbs_solver* s, bool adj, cbs_info* info, bool zero_start
         k_axpy_32_64<<<grid_for(n), 256, 0, s->st>>>(s->x64, s->x32, rn, n);
         CUDA_TRY(cudaGetLastError());
         s->launches += 1;
-        apply_operator<double>(s, adj, INV_RESID);
+        apply_residual<double>(s, adj);
         read_red(s, r);
         info->residual_checks++;
         rn2 = r[0];
@@ -994,7 +972,7 @@ cbs_status solve_common(cbs_solver* s, const void* src, void* field, const void*
         if (herr != 0) {
             CUDA_TRY(cudaMemsetAsync(s->errword, 0, sizeof(int), s->st));
             CUDA_TRY(cudaStreamSynchronize(s->st));
-            st = herr == kErrTileAlign ? CBS_ECUDA : CBS_ETIMEOUT;
+            st = CBS_ETIMEOUT;
         }
         float ms = 0;
         CUDA_TRY(cudaEventElapsedTime(&ms, s->ev0, s->ev1));
@@ -1009,7 +987,6 @@ cbs_status solve_common(cbs_solver* s, const void* src, void* field, const void*
         if (st == CBS_ENOCONV) s->err = "max_iter reached before tol";
         if (st == CBS_EDIVERGED) s->err = "iteration produced a non-finite value";
         if (st == CBS_ETIMEOUT) s->err = "a bulk copy did not complete within its wait limit";
-        if (herr == kErrTileAlign) s->err = "shared-memory tile not 128-byte aligned for tensor copies";
         return st;
     } catch (const CudaError& e) {
         return set_err(s, CBS_ECUDA, std::string("CUDA error ") + cudaGetErrorString(e.e) + " in " + e.what);
@@ -1094,8 +1071,8 @@ std::mutex g_l2_mu;
 int g_l2_users = 0;
 size_t g_l2_limit0 = 0;
 
-// Keep the float32 work array resident in L2 across the five kernels of an
-// iteration: an access-policy window marks it persisting (the others stream).
+// Keep the float32 work fields resident in L2 across the kernels of an
+// iteration: an access-policy window marks them persisting (the others stream).
 // The persisting-L2 limit is a property of this process's CUDA context (it
 // ends with the context); it is raised only up to the device maximum.
 void set_l2_window(cbs_solver* s, void* base, size_t bytes)
@@ -1133,92 +1110,37 @@ void set_l2_window(cbs_solver* s, void* base, size_t bytes)
     cudaGetLastError();
 }
 
-// cuTensorMapEncodeTiled, looked up once through the runtime (no link against the driver library)
-PFN_cuTensorMapEncodeTiled_v12000 tensor_map_encoder()
+using cd = std::complex<double>;
+
+// per-axis tables of (L+I)^-1 (top of born.cuh): tm = -(c1 / c2) conj(t), td = -Pu c1 / (l1 l2) t, forward and with
+// the constants conjugated for the adjoint
+void green_tables(cbs_solver* s, TablePack& pack)
 {
-    static PFN_cuTensorMapEncodeTiled_v12000 fn = []() -> PFN_cuTensorMapEncodeTiled_v12000 {
-        void* p = nullptr;
-        cudaDriverEntryPointQueryResult q;
-        if (cudaGetDriverEntryPointByVersion("cuTensorMapEncodeTiled", &p, 12000, cudaEnableDefault, &q) != cudaSuccess ||
-            q != cudaDriverEntryPointSuccess) {
-            cudaGetLastError();
-            return nullptr;
+    const double l1 = s->lam1, l2 = s->lam2;
+    const cd a1l(s->a1r + l1, s->a1i);
+    for (int adj = 0; adj < 2; ++adj) {
+        cd c1(0.0, std::sqrt(l1 * l2)), c2 = l2 * a1l, pu = l1 / a1l;
+        if (adj) { c1 = std::conj(c1); c2 = std::conj(c2); pu = std::conj(pu); }
+        const cd fm = -(c1 / c2), fd = -pu * c1 / (l1 * l2);
+        for (int a = 0; a < s->D; ++a) {
+            const int n = s->n[a];
+            std::vector<double2> m(n), d(n);
+            std::vector<float2> m32(n), d32(n);
+            for (int i = 0; i < n; ++i) {
+                const cd t(s->kt_host[a][i].x, s->kt_host[a][i].y);
+                const cd tm = fm * std::conj(t), td = fd * t;
+                m[i] = make_double2(tm.real(), tm.imag());
+                d[i] = make_double2(td.real(), td.imag());
+                m32[i] = make_float2((float)tm.real(), (float)tm.imag());
+                d32[i] = make_float2((float)td.real(), (float)td.imag());
+            }
+            pack.add(&s->tm64[adj][a], m);
+            pack.add(&s->td64[adj][a], d);
+            pack.add(&s->tm32[adj][a], m32);
+            pack.add(&s->td32[adj][a], d32);
         }
-        return reinterpret_cast<PFN_cuTensorMapEncodeTiled_v12000>(p);
-    }();
-    return fn;
-}
-
-// Tensor-copy descriptor of the float32 work field for the tile-staged last-axis kernel: the field
-// [C][n2][n1][n0] seen as {n0, n1, C*n2} 8-byte elements, box {COLS, 1, n2}.  The tile kernel is
-// opt-in (environment variable CBS_TILE_LAST): on GB300 it measured no faster than the register
-// kernel (41.0 us at 128^3) and slower at 64^3 and 256^3.  Leaves tile_field null (register kernel)
-// when not asked for, when the sizes do not qualify, or when the descriptor cannot be made.
-template <typename R> void fill_tile_map(cbs_solver* s, Plan<R>& P, const void* field)
-{
-    P.tile_field = nullptr;
-    const int n2 = s->n[2];
-    if (s->D != 3 || field == nullptr || !tile_ok<R>(n2) || s->n[0] % cols_tile<R>(n2) != 0) return;
-    if (std::getenv("CBS_TILE_LAST") == nullptr) return;
-    auto enc = tensor_map_encoder();
-    if (!enc) return;
-    const cuuint64_t gdim[3] = {(cuuint64_t)s->n[0], (cuuint64_t)s->n[1], (cuuint64_t)s->C * n2};
-    const cuuint64_t gstride[2] = {(cuuint64_t)s->n[0] * sizeof(cplx<R>),
-                                   (cuuint64_t)s->n[0] * s->n[1] * sizeof(cplx<R>)};
-    const cuuint32_t box[3] = {(cuuint32_t)cols_tile<R>(n2), 1u, (cuuint32_t)n2};
-    const cuuint32_t estr[3] = {1u, 1u, 1u};
-    static_assert(sizeof(cplx<R>) == 8, "the descriptor treats one complex value as one 8-byte element");
-    const CUresult r = enc(&P.tmap_last, CU_TENSOR_MAP_DATA_TYPE_UINT64, 3, const_cast<void*>(field), gdim, gstride,
-                           box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE,
-                           CU_TENSOR_MAP_L2_PROMOTION_L2_128B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
-    if (r == CUDA_SUCCESS) P.tile_field = field;
-    TRACE("tile map for the last axis: %s", r == CUDA_SUCCESS ? "yes" : "no");
-}
-
-// The float32 last-axis step runs on a cluster of C CTAs (one component each) for 2D grids whose last axis
-// has 2048 points: measured on GB300, 2048^2 takes 142.5 instead of 170.7 us (8-column tiles, 64-byte rows,
-// instead of 2-column tiles holding all three components).  Elsewhere the one-CTA kernel is faster (128^3:
-// 37.9 against 53.5 us; 512^3: 3.25 against 4.26 ms; 1024^2: 32.9 against 34.9 us).  CBS_LAST_CLUSTER=1 /
-// =0 forces it on (extents 64 .. 2048) / off.
-bool last_cluster_preferred(const cbs_solver* s)
-{
-    const int nl = s->n[s->D - 1];
-    if (!last_cluster_ok<float>(nl)) return false;
-    const char* e = std::getenv("CBS_LAST_CLUSTER");
-    if (e != nullptr) return e[0] == '1';
-    return s->D == 2 && nl >= 2048;
-}
-
-// Tensor-copy descriptor and persistent grid of the pipelined strided-axis kernel (3D float32, n1 <= 256,
-// n0 % COLS == 0): the field as {n0, n1, C*n2} 8-byte elements, box {COLS, n1, 1}.  Opt-in with
-// CBS_AXIS_PIPE=1.
-template <typename R> void fill_axis_map(cbs_solver* s, Plan<R>& P, const void* field)
-{
-    P.axis_field = nullptr;
-    P.axis_grid = 0;
-    const int n1 = s->n[1];
-    if (s->D != 3 || field == nullptr || !axis_pipe_ok<R>(n1) || s->n[0] % cols_axis<R>(n1) != 0) return;
-    if (std::getenv("CBS_AXIS_PIPE") == nullptr) return;
-    auto enc = tensor_map_encoder();
-    if (!enc) return;
-    int dev = 0, sms = 0;
-    if (cudaGetDevice(&dev) != cudaSuccess || cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) {
-        cudaGetLastError();
-        return;
     }
-    const int per_sm = axis_pipe_blocks_per_sm<R>(n1);
-    if (per_sm <= 0) return;
-    const cuuint64_t gdim[3] = {(cuuint64_t)s->n[0], (cuuint64_t)n1, (cuuint64_t)s->C * s->n[2]};
-    const cuuint64_t gstride[2] = {(cuuint64_t)s->n[0] * sizeof(cplx<R>), (cuuint64_t)s->n[0] * n1 * sizeof(cplx<R>)};
-    const cuuint32_t box[3] = {(cuuint32_t)cols_axis<R>(n1), (cuuint32_t)n1, 1u};
-    const cuuint32_t estr[3] = {1u, 1u, 1u};
-    const CUresult r = enc(&P.tmap_axis, CU_TENSOR_MAP_DATA_TYPE_UINT64, 3, const_cast<void*>(field), gdim, gstride,
-                           box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE,
-                           CU_TENSOR_MAP_L2_PROMOTION_L2_128B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
-    if (r != CUDA_SUCCESS) return;
-    P.axis_field = field;
-    P.axis_grid = sms * per_sm;
-    TRACE("pipelined axis kernel: %d CTAs", P.axis_grid);
+    pack.upload(s);
 }
 
 template <typename R> void fill_plan(cbs_solver* s, Plan<R>& P)
@@ -1233,8 +1155,6 @@ template <typename R> void fill_plan(cbs_solver* s, Plan<R>& P)
         P.M.rs[e] = f ? (const R*)s->rs32[e] : (const R*)s->rs64[e];
         P.M.gc[e] = f ? (const R*)s->gc32[e] : (const R*)s->gc64[e];
         P.M.gs[e] = f ? (const R*)s->gs32[e] : (const R*)s->gs64[e];
-        P.Sy.kt[e] = f ? (const cplx<R>*)s->kt32[e] : (const cplx<R>*)s->kt64[e];
-        P.Sy.k2[e] = f ? (const R*)s->k232[e] : (const R*)s->k264[e];
         P.tw[e] = f ? (const cplx<R>*)s->tw32[e] : (const cplx<R>*)s->tw64[e];
     }
     P.M.kp = f ? (const R*)s->kp32 : (const R*)s->kp64;
@@ -1244,23 +1164,47 @@ template <typename R> void fill_plan(cbs_solver* s, Plan<R>& P)
     P.M.a1i = (R)(s->a1i / s->lam1);
     P.M.a2r = (R)(s->a2r / s->lam2);
     P.M.a2i = (R)(s->a2i / s->lam2);
-    // symbol constants (App. B.1 with a = a1, lambda_0 = lambda1, b = a2, lambda_1 = lambda2)
+    // (L+I)^-1 (App. B.1 with a = a1, lambda_0 = lambda1, b = a2, lambda_1 = lambda2) and L
+    const double l1 = s->lam1, l2 = s->lam2, isq = 1.0 / std::sqrt(l1 * l2);
+    const cd a1l(s->a1r + l1, s->a1i), a2l(s->a2r + l2, s->a2i);
+    auto c = [](cd v) { return mk<cplx<R>, R>((R)v.real(), (R)v.imag()); };
+    for (int adj = 0; adj < 2; ++adj) {
+        auto cj = [&](cd v) { return c(adj ? std::conj(v) : v); };
+        Symbol<R>& Y = P.Sy[adj];
+        Y.Pu = cj(l1 / a1l);
+        Y.c3 = cj(a1l * a2l);
+        Y.cs = cj(l2 * a1l / (double)s->N);
+        LOp<R>& L = P.L[adj];
+        L.la1 = cj(cd(s->a1r / l1, s->a1i / l1));
+        L.la2 = cj(cd(s->a2r / l2, s->a2i / l2));
+        for (int e = 0; e < 3; ++e) {
+            Y.tm[e] = f ? (const cplx<R>*)s->tm32[adj][e] : (const cplx<R>*)s->tm64[adj][e];
+            Y.td[e] = f ? (const cplx<R>*)s->td32[adj][e] : (const cplx<R>*)s->td64[adj][e];
+            Y.k2[e] = f ? (const R*)s->k232[e] : (const R*)s->k264[e];
+            L.kt[e] = f ? (const cplx<R>*)s->kt32[e] : (const cplx<R>*)s->kt64[e];
+            L.g[e] = (R)((adj ? -isq : isq) / s->n[e]);
+        }
+    }
+}
+
+// constants of the comparison build's symbol kernel
+BaseSymbol base_symbol(cbs_solver* s, bool adj)
+{
     const double l1 = s->lam1, l2 = s->lam2;
-    const double apr = s->a1r + l1, api = s->a1i;   // a1 + lambda1
-    const double bpr = s->a2r + l2, bpi = s->a2i;   // a2 + lambda2
-    const double den = apr * apr + api * api;
-    const double Pr = l1 * apr / den, Pi = -l1 * api / den;  // lambda1 / (a1 + lambda1)
-    const double scale = 1.0 / (double)s->N;
-    const double sq = std::sqrt(l1 * l2);
-    P.Sy.Pu = mk<cplx<R>, R>((R)Pr, (R)Pi);
-    P.Sy.P = mk<cplx<R>, R>((R)(Pr * scale), (R)(Pi * scale));
-    P.Sy.c1 = mk<cplx<R>, R>((R)0, (R)sq);
-    P.Sy.c2 = mk<cplx<R>, R>((R)(l2 * apr), (R)(l2 * api));
-    P.Sy.c3 = mk<cplx<R>, R>((R)(apr * bpr - api * bpi), (R)(apr * bpi + api * bpr));
-    P.Sy.la1 = mk<cplx<R>, R>((R)(s->a1r / l1), (R)(s->a1i / l1));
-    P.Sy.la2 = mk<cplx<R>, R>((R)(s->a2r / l2), (R)(s->a2i / l2));
-    P.Sy.isq = (R)(1.0 / sq);
-    P.Sy.scale = (R)scale;
+    const cd a1l(s->a1r + l1, s->a1i), a2l(s->a2r + l2, s->a2i), scale(1.0 / (double)s->N);
+    auto c = [&](cd v) { return adj ? make_float2((float)v.real(), (float)-v.imag()) : make_float2((float)v.real(), (float)v.imag()); };
+    BaseSymbol Y;
+    Y.P = c(l1 / a1l * scale);
+    Y.Pu = c(l1 / a1l);
+    Y.c1 = c(cd(0.0, std::sqrt(l1 * l2)));
+    Y.c2 = c(l2 * a1l);
+    Y.c3 = c(a1l * a2l);
+    Y.scale = (float)scale.real();
+    for (int e = 0; e < 3; ++e) {
+        Y.kt[e] = s->kt32[e];
+        Y.k2[e] = s->k232[e];
+    }
+    return Y;
 }
 
 // Failure-detection self-test: thread 0 arms the barrier for two elements but
@@ -1387,6 +1331,7 @@ cbs_status solver_create(const cbs_grid* grid, double dx, double omega, const do
         const long long N = s->N;
         const int D = s->D;
         // per-axis tables (host, float64): gamma, wavenumbers, twiddles
+        TablePack pack, green_pack;  // alive until the last synchronisation below
         for (int a = 0; a < 3; ++a) {
             const int n = s->n[a];
             std::vector<double> gc(n, 0.0), gs(n, 0.0), k2(n, 0.0);
@@ -1412,18 +1357,19 @@ cbs_status solver_create(const cbs_grid* grid, double dx, double omega, const do
                 kt32[i] = make_float2((float)kt[i].x, (float)kt[i].y);
                 tw32[i] = make_float2((float)tw[i].x, (float)tw[i].y);
             }
-            s->gc64[a] = dalloc<double>(s, n); upload(s, s->gc64[a], gc);
-            s->gs64[a] = dalloc<double>(s, n); upload(s, s->gs64[a], gs);
-            s->k264[a] = dalloc<double>(s, n); upload(s, s->k264[a], k2);
-            s->kt64[a] = dalloc<double2>(s, n); upload(s, s->kt64[a], kt);
-            s->tw64[a] = dalloc<double2>(s, n); upload(s, s->tw64[a], tw);
-            s->gc32[a] = dalloc<float>(s, n); upload(s, s->gc32[a], gc32);
-            s->gs32[a] = dalloc<float>(s, n); upload(s, s->gs32[a], gs32);
-            s->k232[a] = dalloc<float>(s, n); upload(s, s->k232[a], k232);
-            s->kt32[a] = dalloc<float2>(s, n); upload(s, s->kt32[a], kt32);
-            s->tw32[a] = dalloc<float2>(s, n); upload(s, s->tw32[a], tw32);
-            CUDA_TRY(cudaStreamSynchronize(s->st));  // host vectors go out of scope
+            s->kt_host[a] = kt;
+            pack.add(&s->gc64[a], gc);
+            pack.add(&s->gs64[a], gs);
+            pack.add(&s->k264[a], k2);
+            pack.add(&s->kt64[a], kt);
+            pack.add(&s->tw64[a], tw);
+            pack.add(&s->gc32[a], gc32);
+            pack.add(&s->gs32[a], gs32);
+            pack.add(&s->k232[a], k232);
+            pack.add(&s->kt32[a], kt32);
+            pack.add(&s->tw32[a], tw32);
         }
+        pack.upload(s);
         SetupIn si;
         si.colloc = o.grid_kind == CBS_GRID_COLLOCATED ? 1 : 0;
         si.D = D; si.n0 = s->n[0]; si.n1 = s->n[1]; si.n2 = s->n[2]; si.N = N; si.omega = omega;
@@ -1522,24 +1468,15 @@ cbs_status solver_create(const cbs_grid* grid, double dx, double omega, const do
             s->x32 = dalloc<float2>(s, n);
             s->y32 = dalloc<float2>(s, n);
             s->w32 = dalloc<float2>(s, n);
-            if (std::getenv("CBS_NO_L2_WINDOW") == nullptr) set_l2_window(s, s->w32, (size_t)n * sizeof(float2));
+            // (slot 0 of w carries no field)
+            if (std::getenv("CBS_NO_L2_WINDOW") == nullptr)
+                set_l2_window(s, s->w32 + N, (size_t)D * N * sizeof(float2));
         }
         TRACE("create: plans");
+        green_tables(s, green_pack);
         fill_plan<double>(s, s->P64);
         fill_plan<float>(s, s->P32);
-        fill_tile_map<float>(s, s->P32, s->w32);
-        fill_axis_map<float>(s, s->P32, s->w32);
-        // CBS_PLANE=1 / CBS_NO_PLANE=1 force the plane kernels on (where they exist) / off
-        s->P32.plane = o.precision != CBS_FP64 && std::getenv("CBS_NO_PLANE") == nullptr &&
-                       (std::getenv("CBS_PLANE") != nullptr ? plane_ok<float>(s->P32) : plane_preferred<float>(s->P32));
-        s->P32.last_cluster = o.precision != CBS_FP64 && last_cluster_preferred(s);
-        // CBS_PLANE_CL=4: four CTAs per x-y plane (quarter planes) in place of a pair
-        {
-            const char* e = std::getenv("CBS_PLANE_CL");
-            s->P32.plane_cl = (e != nullptr && e[0] == '4') ? 4 : 2;
-        }
-        const int nb = std::max(std::max(rows_blocks<double>(s->P64), rows_blocks<float>(s->P32)),
-                                std::max(grid_for(n), plane_blocks<float>(s->P32)));
+        const int nb = std::max(std::max(rows_blocks<double>(s->P64), rows_blocks<float>(s->P32)), grid_for(n));
         s->npart = nb;
         s->kslots = std::min(o.check_every, kHostBuf / 2);
         TRACE("create: partials %d x %d", nb, s->kslots);
@@ -1550,15 +1487,6 @@ cbs_status solver_create(const cbs_grid* grid, double dx, double omega, const do
         CUDA_TRY(cudaMemsetAsync(s->errword, 0, sizeof(int), s->st));
         s->P64.err = s->errword;
         s->P32.err = s->errword;
-        // one kernel for the update of an iteration and the forward row transform of the next, where the rows
-        // are bulk-staged; CBS_NO_FUSED_ROWS=1 keeps them apart
-        {
-            const bool off = std::getenv("CBS_NO_FUSED_ROWS") != nullptr;
-            s->P64.fused_rows = !off && fused_rows_ok<double>(s->P64);
-            s->P32.fused_rows = !off && o.precision != CBS_FP64 && fused_rows_ok<float>(s->P32);
-            const char* v = std::getenv("CBS_FUSED_VAR");  // measured variants of the fused row kernel
-            s->P32.fused_var = (v != nullptr && ((v[0] >= '0' && v[0] <= '3') || v[0] == '6')) ? v[0] - '0' : -1;
-        }
         CUDA_TRY(cudaEventRecord(s->ev1, s->st));
         CUDA_TRY(cudaStreamSynchronize(s->st));
         float ms = 0;
@@ -1594,7 +1522,7 @@ cbs_status residual_norm(cbs_solver* s, const void* field, const void* src, int 
     try {
         begin_call(s);
         prepare(s, src, field, adjoint != 0);
-        apply_operator<double>(s, adjoint != 0, INV_RESID);
+        apply_residual<double>(s, adjoint != 0);
         double r[2];
         read_red(s, r);
         *rel = r[1] > 0 ? std::sqrt(r[0] / r[1]) : 0.0;
@@ -1623,8 +1551,8 @@ cbs_status born_iterate(cbs_solver* s, const void* y, void* x, int n_iter, int a
         int done = 0;
         while (done < n_iter) {
             const int blk = std::min(s->kslots, n_iter - done);
-            if (f32) iterate_block<float>(s, blk, adjoint != 0);
-            else iterate_block<double>(s, blk, adjoint != 0);
+            if (f32) iterate_block<float>(s, blk, adjoint != 0, incr != nullptr);
+            else iterate_block<double>(s, blk, adjoint != 0, incr != nullptr);
             if (incr) {
                 CUDA_TRY(cudaMemcpyAsync(s->host_red, s->hist, 2 * blk * sizeof(double), cudaMemcpyDeviceToHost, s->st));
                 CUDA_TRY(cudaStreamSynchronize(s->st));
@@ -1655,13 +1583,17 @@ cbs_status green_apply(cbs_solver* s, const void* in, void* out, int adjoint)
         if (s->opt.precision != CBS_FP64) {
             k_cast_64_32<<<grid_for(n), 256, 0, s->st>>>((const double2*)in, s->x32, 1.0, n);
             CUDA_TRY(cudaGetLastError());
-            apply_green<float>(s, adjoint != 0);
+            CUDA_TRY(launch_green<float>(s->P32, s->x32, s->w32, adjoint != 0, s->st));
             k_cast_32_64<<<grid_for(n), 256, 0, s->st>>>(s->w32, (double2*)out, n);
             CUDA_TRY(cudaGetLastError());
         } else {
-            CUDA_TRY(cudaMemcpyAsync(s->x64, in, n * sizeof(double2), cudaMemcpyDeviceToDevice, s->st));
-            apply_green<double>(s, adjoint != 0);
-            CUDA_TRY(cudaMemcpyAsync(out, s->w64, n * sizeof(double2), cudaMemcpyDeviceToDevice, s->st));
+            // straight from the caller's buffer into the caller's buffer, unless they share memory
+            const double2* x = (const double2*)in;
+            if (overlap(in, out, n * sizeof(double2))) {
+                CUDA_TRY(cudaMemcpyAsync(s->x64, in, n * sizeof(double2), cudaMemcpyDeviceToDevice, s->st));
+                x = s->x64;
+            }
+            CUDA_TRY(launch_green<double>(s->P64, x, (double2*)out, adjoint != 0, s->st));
         }
         CUDA_TRY(cudaStreamSynchronize(s->st));
         return CBS_OK;
@@ -1677,9 +1609,12 @@ cbs_status operator_apply(cbs_solver* s, const void* x, void* out, int adjoint)
     try {
         begin_call(s);
         const long long n = field_len(s);
-        CUDA_TRY(cudaMemcpyAsync(s->x64, x, n * sizeof(double2), cudaMemcpyDeviceToDevice, s->st));
-        apply_operator<double>(s, adjoint != 0, INV_APPLY);
-        CUDA_TRY(cudaMemcpyAsync(out, s->w64, n * sizeof(double2), cudaMemcpyDeviceToDevice, s->st));
+        const double2* xi = (const double2*)x;
+        if (overlap(x, out, n * sizeof(double2))) {
+            CUDA_TRY(cudaMemcpyAsync(s->x64, x, n * sizeof(double2), cudaMemcpyDeviceToDevice, s->st));
+            xi = s->x64;
+        }
+        CUDA_TRY(launch_operator<double>(s->P64, xi, nullptr, (double2*)out, OP_APPLY, adjoint != 0, s->partials, s->st));
         CUDA_TRY(cudaStreamSynchronize(s->st));
         return CBS_OK;
     } catch (const CudaError& e) {
@@ -1758,15 +1693,10 @@ cbs_status solver_time_kernels(cbs_solver* s, const void* y, void* x, int n_iter
     if (!s) return CBS_EINVAL;
     if (!y || !x || n_iter <= 0 || !ms || !nk) return set_err(s, CBS_EINVAL, "bad argument");
     const bool f32 = s->opt.precision != CBS_FP64;
-    const char* kn3[5] = {"rows_fwd", "axis_fwd", "last_symbol", "axis_inv", "rows_inv"};
-    const char* kn2[3] = {"rows_fwd", "last_symbol", "rows_inv"};
-    const char* knp[3] = {"plane_fwd", "last_symbol", "plane_inv"};
-    const char* knf3[4] = {"axis_fwd", "last_symbol", "axis_inv", "rows_inv_fwd"};
-    const char* knf2[2] = {"last_symbol", "rows_inv_fwd"};
-    const bool plane = f32 && s->P32.plane;
-    const bool fused = !plane && (f32 ? s->P32.fused_rows : s->P64.fused_rows);
-    const int K = fused ? (s->D == 3 ? 4 : 2) : ((s->D == 3 && !plane) ? 5 : 3);
-    const char** kn = fused ? (s->D == 3 ? knf3 : knf2) : (plane ? knp : (s->D == 3 ? kn3 : kn2));
+    const char* kn3[4] = {"axis_merge", "last_solve", "axis_split", "rows_update"};
+    const int K = s->D == 3 ? 4 : 2;
+    const char* kn2[2] = {"last_solve", "rows_update"};
+    const char** kn = s->D == 3 ? kn3 : kn2;
     try {
         begin_call(s);
         const long long n = field_len(s);
@@ -1780,68 +1710,29 @@ cbs_status solver_time_kernels(cbs_solver* s, const void* y, void* x, int n_iter
         std::vector<cudaEvent_t> ev(K + 1);
         for (auto& e : ev) CUDA_TRY(cudaEventCreate(&e));
         std::vector<double> acc(K, 0.0);
-        // fused rows: the forward row kernel runs once before the timed iterations, each of which is then the
-        // strided-axis and last-axis kernels and the fused update + next forward row kernel
-        if (fused) {
-            if (f32) CUDA_TRY(launch_rows_fwd<float>(s->P32, s->x32, s->y32, s->w32, FWD_BORN, 0, s->st));
-            else CUDA_TRY(launch_rows_fwd<double>(s->P64, s->x64, s->y64, s->w64, FWD_BORN, 0, s->st));
-        }
-        // one untimed iteration first: the first launch of each kernel in a process also loads it
-        for (int it = -1; it < n_iter; ++it) {
-            int k = 0;
-            auto mark = [&]() { CUDA_TRY(cudaEventRecord(ev[k++], s->st)); };
-            mark();
-            if (fused) {
-                auto one = [&](auto& P, auto* x, auto* y, auto* w, auto nu) {
-                    if (s->D == 3) { CUDA_TRY(launch_axis(P, w, -1, s->st)); mark(); }
-                    CUDA_TRY(launch_last(P, w, SYM_GREEN, s->st)); mark();
-                    if (s->D == 3) { CUDA_TRY(launch_axis(P, w, +1, s->st)); mark(); }
-                    CUDA_TRY(launch_rows_inv_fwd(P, x, y, w, 0, nu, s->partials, s->st)); mark();
-                };
-                if (f32) one(s->P32, s->x32, s->y32, s->w32, (float)s->opt.nu);
-                else one(s->P64, s->x64, s->y64, s->w64, s->opt.nu);
+        // the forward row kernel runs once before the timed iterations, each of which is then the strided-axis kernels
+        // and the update + next forward row kernel; one untimed iteration first: the first launch of each kernel in
+        // a process also loads it
+        auto timed = [&](auto& P, auto* x, auto* y, auto* w, auto nu) {
+            CUDA_TRY(launch_rows(P, x, y, w, ROWS_FWD, 0, nu, s->partials, s->st));
+            for (int it = -1; it < n_iter; ++it) {
+                int k = 0;
+                auto mark = [&]() { CUDA_TRY(cudaEventRecord(ev[k++], s->st)); };
+                mark();
+                if (s->D == 3) { CUDA_TRY(launch_axis(P, w, -1, 0, s->st)); mark(); }
+                CUDA_TRY(launch_last(P, w, 0, s->st)); mark();
+                if (s->D == 3) { CUDA_TRY(launch_axis(P, w, +1, 0, s->st)); mark(); }
+                CUDA_TRY(launch_rows(P, x, y, w, ROWS_FUSED, 0, nu, s->partials, s->st)); mark();
                 CUDA_TRY(cudaStreamSynchronize(s->st));
                 for (int j = 0; j < K && it >= 0; ++j) {
-                    float tj = 0;
-                    CUDA_TRY(cudaEventElapsedTime(&tj, ev[j], ev[j + 1]));
-                    acc[j] += tj;
+                    float t = 0;
+                    CUDA_TRY(cudaEventElapsedTime(&t, ev[j], ev[j + 1]));
+                    acc[j] += t;
                 }
-                continue;
             }
-            if (f32) {
-                Plan<float>& P = s->P32;
-                if (plane) {
-                    CUDA_TRY(launch_plane_fwd<float>(P, s->x32, s->y32, s->w32, 0, s->st)); mark();
-                    CUDA_TRY(launch_last<float>(P, s->w32, SYM_GREEN, s->st)); mark();
-                    CUDA_TRY(launch_plane_inv<float>(P, s->x32, s->w32, 0, (float)s->opt.nu, s->partials, s->st)); mark();
-                    CUDA_TRY(cudaStreamSynchronize(s->st));
-                    for (int j = 0; j < K && it >= 0; ++j) {
-                        float tj = 0;
-                        CUDA_TRY(cudaEventElapsedTime(&tj, ev[j], ev[j + 1]));
-                        acc[j] += tj;
-                    }
-                    continue;
-                }
-                CUDA_TRY(launch_rows_fwd<float>(P, s->x32, s->y32, s->w32, FWD_BORN, 0, s->st)); mark();
-                if (s->D == 3) { CUDA_TRY(launch_axis<float>(P, s->w32, -1, s->st)); mark(); }
-                CUDA_TRY(launch_last<float>(P, s->w32, SYM_GREEN, s->st)); mark();
-                if (s->D == 3) { CUDA_TRY(launch_axis<float>(P, s->w32, +1, s->st)); mark(); }
-                CUDA_TRY(launch_rows_inv<float>(P, s->x32, s->y32, s->w32, INV_BORN, 0, (float)s->opt.nu, s->partials, s->st)); mark();
-            } else {
-                Plan<double>& P = s->P64;
-                CUDA_TRY(launch_rows_fwd<double>(P, s->x64, s->y64, s->w64, FWD_BORN, 0, s->st)); mark();
-                if (s->D == 3) { CUDA_TRY(launch_axis<double>(P, s->w64, -1, s->st)); mark(); }
-                CUDA_TRY(launch_last<double>(P, s->w64, SYM_GREEN, s->st)); mark();
-                if (s->D == 3) { CUDA_TRY(launch_axis<double>(P, s->w64, +1, s->st)); mark(); }
-                CUDA_TRY(launch_rows_inv<double>(P, s->x64, s->y64, s->w64, INV_BORN, 0, s->opt.nu, s->partials, s->st)); mark();
-            }
-            CUDA_TRY(cudaStreamSynchronize(s->st));
-            for (int j = 0; j < K && it >= 0; ++j) {
-                float t = 0;
-                CUDA_TRY(cudaEventElapsedTime(&t, ev[j], ev[j + 1]));
-                acc[j] += t;
-            }
-        }
+        };
+        if (f32) timed(s->P32, s->x32, s->y32, s->w32, (float)s->opt.nu);
+        else timed(s->P64, s->x64, s->y64, s->w64, s->opt.nu);
         for (auto& e : ev) cudaEventDestroy(e);
         const int m = std::min(K, max_k);
         for (int j = 0; j < m; ++j) ms[j] = acc[j] / n_iter;
@@ -1906,7 +1797,7 @@ cbs_status cufft_baseline_iterate(cbs_solver* s, const void* y, void* x, int n_i
         CUDA_TRY(cudaGetLastError());
         Plan<float>& P = s->P32;
         const int g = grid_for(n), gs = grid_for(s->N);
-        const int mode = adjoint ? SYM_GREEN_ADJ : SYM_GREEN;
+        const BaseSymbol Sy = base_symbol(s, adjoint != 0);
         cufftComplex* w = reinterpret_cast<cufftComplex*>(s->w32);
         CUDA_TRY(cudaEventRecord(s->ev0, s->st));
         for (int it = 0; it < n_iter; ++it) {
@@ -1914,8 +1805,8 @@ cbs_status cufft_baseline_iterate(cbs_solver* s, const void* y, void* x, int n_i
             CUDA_TRY(cudaGetLastError());
             if (cufftExecC2C(s->fft_plan, w, w, CUFFT_FORWARD) != CUFFT_SUCCESS)
                 return set_err(s, CBS_ECUDA, "cufftExecC2C failed");
-            if (s->D == 3) k_base_symbol<float, 4><<<gs, 256, 0, s->st>>>(P.d, P.Sy, s->w32, mode);
-            else k_base_symbol<float, 3><<<gs, 256, 0, s->st>>>(P.d, P.Sy, s->w32, mode);
+            if (s->D == 3) k_base_symbol<4><<<gs, 256, 0, s->st>>>(P.d, Sy, s->w32);
+            else k_base_symbol<3><<<gs, 256, 0, s->st>>>(P.d, Sy, s->w32);
             CUDA_TRY(cudaGetLastError());
             if (cufftExecC2C(s->fft_plan, w, w, CUFFT_INVERSE) != CUFFT_SUCCESS)
                 return set_err(s, CBS_ECUDA, "cufftExecC2C failed");

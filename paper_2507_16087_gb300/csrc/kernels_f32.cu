@@ -1,5 +1,6 @@
-// Launchers of the float32 Born kernels (all supported axis extents).
+// Launchers of the float32 row kernels (all supported x extents).
 #include "launch.cuh"
 namespace cbs {
-CBS_INSTANTIATE_LAUNCHERS(float)
+CBS_AXIS_LAUNCHERS(extern template, float)
+CBS_ROW_LAUNCHERS(template, float)
 }

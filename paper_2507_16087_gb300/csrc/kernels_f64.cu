@@ -1,5 +1,6 @@
-// Launchers of the float64 Born kernels (all supported axis extents).
+// Launchers of the float64 row kernels (all supported x extents).
 #include "launch.cuh"
 namespace cbs {
-CBS_INSTANTIATE_LAUNCHERS(double)
+CBS_AXIS_LAUNCHERS(extern template, double)
+CBS_ROW_LAUNCHERS(template, double)
 }

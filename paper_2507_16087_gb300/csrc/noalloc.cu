@@ -5,10 +5,10 @@
 // not grow the process's device footprint, or processes where the CUDA
 // allocator is locked down.  green_apply_noalloc serves them: the caller
 // passes the input and output buffers, and every other piece of device memory
-// the transform needs (twiddle and wavenumber tables, the inverse-x kernel's
-// per-block norm partials) lives in the file-scope array below.  That array
-// is part of the library image: every GPU that loads the library holds it
-// (kNoAllocScratchDoubles * 8 bytes = 124 KiB) until the process exits.
+// the transform needs (twiddle and wavenumber tables) lives in the file-scope
+// array below.  That array is part of the library image: every GPU that loads
+// the library holds it (kNoAllocScratchDoubles * 8 bytes = 84 KiB) until the
+// process exits.
 //
 // The kernels are the same ones green_apply runs for a solver on the
 // staggered grid (App. B.1, the default grid kind); the output buffer doubles
@@ -17,6 +17,7 @@
 #include <cuda_runtime.h>
 
 #include <cmath>
+#include <complex>
 #include <mutex>
 #include <string>
 
@@ -34,12 +35,11 @@ namespace {
 
 constexpr int kMaxAxis = 512;                    // largest supported extent
 constexpr long long kMaxVoxels = 1LL << 21;      // N <= 2,097,152 (e.g. 128^3, 512 x 64 x 64, 512 x 512)
-constexpr int kMaxPartialBlocks = 4096;          // inverse-x kernel blocks for N <= kMaxVoxels
 constexpr int kTwOff = 0;                                   // double2 tw[3][kMaxAxis]
-constexpr int kKtOff = kTwOff + 3 * kMaxAxis * 2;           // double2 kt[3][kMaxAxis]
-constexpr int kK2Off = kKtOff + 3 * kMaxAxis * 2;           // double  k2[3][kMaxAxis]
-constexpr int kPartOff = kK2Off + 3 * kMaxAxis;             // double  partials[2 * kMaxPartialBlocks]
-constexpr int kNoAllocScratchDoubles = kPartOff + 2 * kMaxPartialBlocks;
+constexpr int kTmOff = kTwOff + 3 * kMaxAxis * 2;           // double2 tm[3][kMaxAxis]: merge factors
+constexpr int kTdOff = kTmOff + 3 * kMaxAxis * 2;           // double2 td[3][kMaxAxis]: split factors
+constexpr int kK2Off = kTdOff + 3 * kMaxAxis * 2;           // double  k2[3][kMaxAxis]
+constexpr int kNoAllocScratchDoubles = kK2Off + 3 * kMaxAxis;
 
 static __device__ __align__(256) double g_noalloc_scratch[kNoAllocScratchDoubles];
 
@@ -70,14 +70,15 @@ cudaError_t scratch_address(double** out)
     return cudaSuccess;
 }
 
-// per-axis twiddles exp(-2 pi i j / n), t = k e^{i k dx/2} and k^2 with
-// k = 2 pi fftfreq(n, dx), written into the scratch tables
-__global__ void k_noalloc_tables(int D, int n0, int n1, int n2, double dx, double* scratch)
+// per-axis twiddles exp(-2 pi i j / n), merge and split factors fm conj(t) and fd t of t = k e^{i k dx/2}, and k^2,
+// with k = 2 pi fftfreq(n, dx), written into the scratch tables
+__global__ void k_noalloc_tables(int n0, int n1, int n2, double dx, double2 fm, double2 fd, double* scratch)
 {
     const int a = blockIdx.y;
     const int n = a == 0 ? n0 : (a == 1 ? n1 : n2);
     double2* tw = reinterpret_cast<double2*>(scratch + kTwOff) + a * kMaxAxis;
-    double2* kt = reinterpret_cast<double2*>(scratch + kKtOff) + a * kMaxAxis;
+    double2* tm = reinterpret_cast<double2*>(scratch + kTmOff) + a * kMaxAxis;
+    double2* td = reinterpret_cast<double2*>(scratch + kTdOff) + a * kMaxAxis;
     double* k2 = scratch + kK2Off + a * kMaxAxis;
     for (int j = blockIdx.x * blockDim.x + threadIdx.x; j < n; j += gridDim.x * blockDim.x) {
         double s, c;
@@ -87,10 +88,10 @@ __global__ void k_noalloc_tables(int D, int n0, int n1, int n2, double dx, doubl
         const double k = 2.0 * 3.14159265358979323846 * (double)f / ((double)n * dx);
         double sh, ch;
         sincos(0.5 * k * dx, &sh, &ch);
-        kt[j] = make_double2(k * ch, k * sh);
+        tm[j] = cmul(fm, make_double2(k * ch, -k * sh));
+        td[j] = cmul(fd, make_double2(k * ch, k * sh));
         k2[j] = k * k;
     }
-    (void)D;
 }
 
 cbs_status fail(cbs_status st, const std::string& msg)
@@ -134,44 +135,27 @@ cbs_status green_apply_noalloc(const cbs_grid* grid, double dx, const double* sc
     P.d.n1 = n[1];
     P.d.n2 = n[2];
     P.d.N = N;
-    const int nblk = rows_blocks<double>(P);
-    if (nblk > kMaxPartialBlocks) return fail(CBS_EINVAL, "grid needs more norm partials than the scratch holds");
+    // (L+I)^-1 constants (App. B.1, a = a1, lambda_0 = lambda1, b = a2, lambda_1 = lambda2; top of born.cuh),
+    // conjugated for the adjoint
+    using cd = std::complex<double>;
+    auto cj = [&](cd v) { return adjoint ? std::conj(v) : v; };
+    auto d2 = [](cd v) { return make_double2(v.real(), v.imag()); };
+    const cd a1l(scalars[0] + l1, scalars[1]), a2l(scalars[2] + l2, scalars[3]);
+    const cd c1 = cj(cd(0.0, std::sqrt(l1 * l2))), c2 = cj(l2 * a1l), pu = cj(l1 / a1l);
+    Symbol<double>& Y = P.Sy[adjoint ? 1 : 0];
+    Y.Pu = d2(pu);
+    Y.c3 = d2(cj(a1l * a2l));
+    Y.cs = d2(c2 / (double)N);
     for (int a = 0; a < 3; ++a) {
         P.tw[a] = reinterpret_cast<const double2*>(scratch + kTwOff) + a * kMaxAxis;
-        P.Sy.kt[a] = reinterpret_cast<const double2*>(scratch + kKtOff) + a * kMaxAxis;
-        P.Sy.k2[a] = scratch + kK2Off + a * kMaxAxis;
-        // the copy / plain modes read the layer tables only as unused row
-        // constants: any readable table of n_a values serves
-        P.M.gc[a] = P.Sy.k2[a];
-        P.M.gs[a] = P.Sy.k2[a];
+        Y.tm[a] = reinterpret_cast<const double2*>(scratch + kTmOff) + a * kMaxAxis;
+        Y.td[a] = reinterpret_cast<const double2*>(scratch + kTdOff) + a * kMaxAxis;
+        Y.k2[a] = scratch + kK2Off + a * kMaxAxis;
     }
-    // (L+I)^-1 symbol constants (App. B.1, a = a1, lambda_0 = lambda1, b = a2, lambda_1 = lambda2)
-    const double apr = scalars[0] + l1, api = scalars[1];
-    const double bpr = scalars[2] + l2, bpi = scalars[3];
-    const double den = apr * apr + api * api;
-    const double Pr = l1 * apr / den, Pi = -l1 * api / den;
-    const double scale = 1.0 / (double)N;
-    const double sq = std::sqrt(l1 * l2);
-    P.Sy.Pu = make_double2(Pr, Pi);
-    P.Sy.P = make_double2(Pr * scale, Pi * scale);
-    P.Sy.c1 = make_double2(0.0, sq);
-    P.Sy.c2 = make_double2(l2 * apr, l2 * api);
-    P.Sy.c3 = make_double2(apr * bpr - api * bpi, apr * bpi + api * bpr);
-    P.Sy.la1 = make_double2(scalars[0] / l1, scalars[1] / l1);
-    P.Sy.la2 = make_double2(scalars[2] / l2, scalars[3] / l2);
-    P.Sy.isq = 1.0 / sq;
-    P.Sy.scale = scale;
-
-    k_noalloc_tables<<<dim3(4, 3), 128, 0, st>>>(grid->ndim, n[0], n[1], n[2], dx, scratch);
+    k_noalloc_tables<<<dim3(4, 3), 128, 0, st>>>(n[0], n[1], n[2], dx, d2(-(c1 / c2)), d2(-pu * c1 / (l1 * l2)), scratch);
     e = cudaGetLastError();
-    const double2* x = static_cast<const double2*>(in);
-    double2* w = static_cast<double2*>(out);
-    double* partials = scratch + kPartOff;
-    if (e == cudaSuccess) e = launch_rows_fwd<double>(P, x, nullptr, w, FWD_COPY, 0, st);
-    if (e == cudaSuccess && P.d.D == 3) e = launch_axis<double>(P, w, -1, st);
-    if (e == cudaSuccess) e = launch_last<double>(P, w, adjoint ? SYM_GREEN_ADJ : SYM_GREEN, st);
-    if (e == cudaSuccess && P.d.D == 3) e = launch_axis<double>(P, w, +1, st);
-    if (e == cudaSuccess) e = launch_rows_inv<double>(P, nullptr, nullptr, w, INV_PLAIN, 0, 0.0, partials, st);
+    if (e == cudaSuccess)
+        e = launch_green<double>(P, static_cast<const double2*>(in), static_cast<double2*>(out), adjoint ? 1 : 0, st);
     if (e == cudaSuccess) e = cudaStreamSynchronize(st);
     if (e != cudaSuccess) return fail(CBS_ECUDA, std::string("CUDA error ") + cudaGetErrorString(e));
     return CBS_OK;
