@@ -38,6 +38,8 @@
 //   v_p   = kp [(gamma + et omega) + i (omega - gamma et)] - a2/lambda2
 // (eq. LV with q = (i omega + gamma)/(rho c^2), c^2 of eq. 118).
 #pragma once
+#include <type_traits>
+
 #include "fft.cuh"
 
 namespace cbs {
@@ -244,15 +246,16 @@ __device__ __forceinline__ void fence_proxy_async_smem() { asm volatile("fence.p
 // ----------------------------------------------------------------- rows
 // One transform unit is one x row of one component, done by T = NX / RX threads; a block holds U units.  Blocks
 // of the first kind (b < npair) take U/2 rows of the pair (p, u_x): units [0, U/2) are the pressure's, the rest
-// u_x's; blocks of the second kind take U rows of one other velocity component.  All of a block's rows are
-// contiguous in each array and are staged by bulk copies on mbarriers (w first, then x and the medium, then y).
-// y lands in w's buffer once the inverse transform has been read out of it (ysep = 0: two field buffers a block,
+// u_x's; blocks of the second kind take U rows of one other velocity component.  The rows are staged by one bulk
+// copy each on mbarriers (w first, then x and the medium, then y) at the pitch of the transform's exchange, so the
+// exchange runs in the staged w row and the rows that share a shared-memory phase lie on different banks.
+// y lands in w's rows once the inverse transform has been read out of them (ysep = 0: two field buffers a block,
 // more blocks an SM) or in a buffer of its own, issued at the start (ysep = 1: small grids, where a block's
 // chain of waits is the time).  The two modes without B (ROWS_COPY, ROWS_GREEN) load straight from global memory.
 template <typename R, int NX, int RX> struct RowCfg {
     static constexpr int T = NX / RX;
-    static constexpr int SL = sm_len<NX, true>();       // row length of the transform's exchange
-    static constexpr bool INPLACE = SL == NX;           // the exchange runs in the staged w rows
+    static constexpr int SL = RowPad<cplx<R>, NX, T>::SL;        // row pitch of the field buffers (values)
+    static constexpr int ML = (SL + 3) / 4 * 4;                  // row pitch of the medium buffers (reals)
     // 64 threads: many small blocks in different phases keep copies in flight (128 threads: 63.8 against 62.1 us at
     // 128^3, 421 against 410 us at 256^3)
     static constexpr int UMAX = 64 / T < 2 ? 2 : 64 / T;
@@ -260,14 +263,34 @@ template <typename R, int NX, int RX> struct RowCfg {
     static constexpr int MAXT = UMAX * T;
     // float32: 128 registers a thread, 168 with 24 values
     static constexpr int MINB = sizeof(R) == 4 ? (RX >= 24 ? 384 / MAXT : 512 / MAXT) : 1;
-    // shared memory of a block of U units
+    // shared memory of a block of U units: x, w (and y), the medium rows (three a pair row), three barriers
     __host__ __device__ static constexpr size_t smem(int U, bool ysep)
     {
-        const size_t E = (size_t)U * NX;
-        return E * sizeof(cplx<R>) * (ysep ? 3 : 2) + (INPLACE ? 0 : (size_t)U * SL * sizeof(cplx<R>)) +
-               E / 2 * 3 * sizeof(R) + 32;
+        return (size_t)U * SL * sizeof(cplx<R>) * (ysep ? 3 : 2) + (size_t)U / 2 * 3 * ML * sizeof(R) + 32;
     }
 };
+
+// B = 1 - v from a voxel's medium values, m0 = rs_c (velocity, m1 = 0) or kp (pressure, m1 = et):
+//   Re B = c.x - m0 (g + m1 omega),  Im B = c.y - m0 (omega - g m1)  with c = 1 + a / lambda; conj for the adjoint
+template <typename R> struct UnitB {
+    R cr, ci, om, so;  // c, omega, sign of the imaginary part times omega
+    R si;              // +1, adjoint -1
+};
+template <typename R> __device__ __forceinline__ UnitB<R> unit_B(const Medium<R>& M, bool pres, bool adj)
+{
+    UnitB<R> u;
+    u.si = adj ? (R)-1 : (R)1;
+    u.cr = (R)1 + (pres ? M.a2r : M.a1r);
+    u.ci = u.si * (pres ? M.a2i : M.a1i);
+    u.om = M.omega;
+    u.so = u.si * M.omega;
+    return u;
+}
+template <bool PAIR, typename R> __device__ __forceinline__ cplx<R> voxel_B(const UnitB<R>& u, R g, R m0, R m1)
+{
+    if constexpr (PAIR) return mk<cplx<R>, R>(fma(-m0, fma(m1, u.om, g), u.cr), fma(-m0, fma(-g * u.si, m1, u.so), u.ci));
+    else return mk<cplx<R>, R>(fma(-m0, g, u.cr), fma(-m0, u.so, u.ci));
+}
 
 template <typename R, int NX, int RX, int MODE>
 __global__ void __launch_bounds__(RowCfg<R, NX, RX>::MAXT, RowCfg<R, NX, RX>::MINB)
@@ -277,24 +300,22 @@ k_rows(Dims d, Medium<R> M, Symbol<R> Sy, cplx<R>* __restrict__ x, const cplx<R>
 {
     using CT = cplx<R>;
     using Cfg = RowCfg<R, NX, RX>;
-    constexpr int T = Cfg::T, SL = Cfg::SL;
+    constexpr int T = Cfg::T, SL = Cfg::SL, ML = Cfg::ML;
     constexpr int np = plan_npass(NX, RX);
-    constexpr bool HAS_W = MODE == ROWS_FUSED || MODE == ROWS_FUSED_NORM || MODE == ROWS_INV || MODE == ROWS_GREEN;
     constexpr bool UPDATE = MODE == ROWS_FUSED || MODE == ROWS_FUSED_NORM || MODE == ROWS_INV;
+    constexpr bool HAS_W = UPDATE || MODE == ROWS_GREEN;
     constexpr bool HAS_B = UPDATE || MODE == ROWS_FWD;  // B, y and the medium
     constexpr bool HAS_FWD = MODE == ROWS_FWD || MODE == ROWS_FUSED || MODE == ROWS_FUSED_NORM || MODE == ROWS_COPY;
     constexpr bool NORM = MODE == ROWS_FUSED_NORM || MODE == ROWS_INV;
     extern __shared__ __align__(128) unsigned char smraw[];
     const int U = blockDim.x / T, H = U >> 1;
-    const int E = U * NX;
+    const int E = U * SL;
     CT* xs = reinterpret_cast<CT*>(smraw);
     CT* ws = xs + E;
-    CT* ex = Cfg::INPLACE ? ws : ws + E;
-    CT* after = Cfg::INPLACE ? ws + E : ex + U * SL;
     const bool yown = UPDATE && ysep != 0;
-    CT* ys = yown ? after : ws;
-    R* ms = reinterpret_cast<R*>(yown ? after + E : after);
-    uint64_t* bar = reinterpret_cast<uint64_t*>(ms + E / 2 * 3);
+    CT* ys = yown ? ws + E : ws;
+    R* ms = reinterpret_cast<R*>(ws + (yown ? 2 * E : E));
+    uint64_t* bar = reinterpret_cast<uint64_t*>(ms + 3 * H * ML);
     const int lu = threadIdx.x / T, t = threadIdx.x % T;
     const long long rpc = d.N / NX;  // rows per component
     const bool pair = (int)blockIdx.x < npair;
@@ -317,42 +338,44 @@ k_rows(Dims d, Medium<R> M, Symbol<R> Sy, cplx<R>* __restrict__ x, const cplx<R>
     constexpr int nbar = UPDATE ? 3 : 1;
     const long long v0 = row0 * NX;  // first voxel of the block's rows
     const int cs = pair ? d.D : c;   // component (slot) of the block's first array
+    constexpr uint32_t FB = NX * sizeof(CT), MB = NX * sizeof(R);
+    // rows of one array into consecutive buffer rows, one copy a row, the copies spread over the block's threads
+    auto rows_in = [&](auto* dst, const auto* src, int pitch, uint32_t bytes, uint64_t* on) {
+        for (int k = threadIdx.x; k < nrow; k += blockDim.x) bulk_g2s(dst + k * pitch, src + (long long)k * NX, bytes, on);
+    };
+    auto y_in = [&](uint64_t* on) {
+        rows_in(ys, y + (long long)cs * d.N + v0, SL, FB, on);
+        if (pair) rows_in(ys + H * SL, y + v0, SL, FB, on);
+    };
     if constexpr (HAS_B) {
-        if (threadIdx.x == 0)
+        if (threadIdx.x == 0) {
+            const uint32_t fb = (uint32_t)nrow * FB, mb = (uint32_t)nrow * MB, two = pair ? 2u : 1u;
             for (int k = 0; k < nbar; ++k) mbar_init(bar + k, 1);
+            if constexpr (UPDATE) {
+                mbar_expect_tx(bar, fb);
+                mbar_expect_tx(bar + 1, two * fb + (pair ? 3u : 1u) * mb);
+                mbar_expect_tx(bar + 2, two * fb);
+            } else {
+                mbar_expect_tx(bar, 2u * two * fb + (pair ? 3u : 1u) * mb);
+            }
+        }
         __syncthreads();
-    }
-    if (HAS_B && threadIdx.x == 0) {
-        const uint32_t fb = (uint32_t)nrow * NX * sizeof(CT), mb = (uint32_t)nrow * NX * sizeof(R);
-        uint64_t* bx = bar;
-        if constexpr (UPDATE) {
-            mbar_expect_tx(bar, fb);
-            bulk_g2s(ws, w + (long long)cs * d.N + v0, fb, bar);
-            bx = bar + 1;
-        }
-        const uint32_t two = pair ? 2u : 1u;
-        constexpr bool y_now = MODE == ROWS_FWD;
-        mbar_expect_tx(bx, (y_now ? 2u : 1u) * two * fb + (pair ? 3u : 1u) * mb);
-        bulk_g2s(xs, x + (long long)cs * d.N + v0, fb, bx);
+        if constexpr (UPDATE) rows_in(ws, w + (long long)cs * d.N + v0, SL, FB, bar);
+        uint64_t* bx = UPDATE ? bar + 1 : bar;
+        rows_in(xs, x + (long long)cs * d.N + v0, SL, FB, bx);
         if (pair) {
-            bulk_g2s(xs + H * NX, x + v0, fb, bx);
-            bulk_g2s(ms, M.kp + v0, mb, bx);
-            bulk_g2s(ms + H * NX, M.et + v0, mb, bx);
-            bulk_g2s(ms + 2 * H * NX, M.rs[0] + v0, mb, bx);
+            rows_in(xs + H * SL, x + v0, SL, FB, bx);
+            rows_in(ms, M.kp + v0, ML, MB, bx);
+            rows_in(ms + H * ML, M.et + v0, ML, MB, bx);
+            rows_in(ms + 2 * H * ML, M.rs[0] + v0, ML, MB, bx);
         } else {
-            bulk_g2s(ms, (c == 1 ? M.rs[1] : M.rs[2]) + v0, mb, bx);
+            rows_in(ms, (c == 1 ? M.rs[1] : M.rs[2]) + v0, ML, MB, bx);
         }
-        if (y_now || yown) {
-            uint64_t* by = y_now ? bx : bar + 2;
-            if (!y_now) mbar_expect_tx(by, two * fb);
-            bulk_g2s(ys, y + (long long)cs * d.N + v0, fb, by);
-            if (pair) bulk_g2s(ys + H * NX, y + v0, fb, by);
-        }
+        if (!UPDATE || yown) y_in(UPDATE ? bar + 2 : bar);
     }
     TwCache<NX, RX, CT> tc;
     tw_load<NX, RX, T>(tc, t, tw);
     const long long rest = row0 + (valid ? lrow : 0);
-    const int i1 = (int)(rest % d.n1), i2 = (int)(rest / d.n1);
     const long long fbase = (long long)c * d.N + rest * NX;
     // a timed-out wait records the error, lets the block's copies land and leaves; the decision is block-uniform
     auto lost = [&](int k) -> bool {
@@ -363,70 +386,83 @@ k_rows(Dims d, Medium<R> M, Symbol<R> Sy, cplx<R>* __restrict__ x, const cplx<R>
         }
         return true;
     };
-    RowB<R> rb{};
-    if constexpr (HAS_B) rb = row_B(M, d.D, c, i1, i2, 0);
-    auto B_at = [&](int i0) -> CT {
-        const int m = lrow * NX + i0;
-        const R g = __ldg(rb.g0 + i0) + rb.grest;
-        return born_B_vals(M, pres, g, isx ? ms[2 * H * NX + m] : ms[m], pres ? ms[H * NX + m] : (R)0, adj != 0);
+    CT* row = ws + lu * SL;  // this unit's row: staged w (or y), and its exchange
+    const CT* xr = xs + lu * SL + t;
+    const CT* yr = ys + lu * SL + t;
+    const R* m0r = ms + (isx ? 2 * H + lrow : lrow) * ML + t;
+    const R* m1r = ms + (H + lrow) * ML + t;
+    UnitB<R> ub{};
+    const R* g0 = nullptr;
+    R grest = (R)0;
+    if constexpr (HAS_B) {
+        const RowB<R> rb = row_B(M, d.D, c, (int)(rest % d.n1), (int)(rest / d.n1), 0);
+        ub = unit_B(M, pres, adj != 0);
+        g0 = rb.g0 + t;
+        grest = rb.grest;
+    }
+    const R has_et = pres ? (R)1 : (R)0;
+    auto B_at = [&](int o, auto is_pair) -> CT {  // o: compile-time offset from t
+        const R g = __ldg(g0 + o) + grest;
+        if constexpr (decltype(is_pair)::value) return voxel_B<true>(ub, g, m0r[o], has_et * m1r[o]);
+        else return voxel_B<false>(ub, g, m0r[o], (R)0);
     };
     CT v[RX];
     if constexpr (HAS_W) {
         // u_x's units read the pressure's row too
-        const CT* wr = ws + (size_t)lrow * NX;
+        const CT* wr;
         if constexpr (UPDATE) {
             if (lost(0)) return;
+            wr = ws + lrow * SL + t;
         } else {
-            wr = w + (long long)cs * d.N + rest * NX;
+            wr = w + (long long)cs * d.N + rest * NX + t;
         }
 #pragma unroll
-        for (int s = 0; s < RX; ++s) v[s] = wr[t + T * slot_q<NX, RX, 0>(s)];
+        for (int s = 0; s < RX; ++s) v[s] = wr[T * slot_q<NX, RX, 0>(s)];
         if (pair) {
             if (isx) {
 #pragma unroll
                 for (int s = 0; s < RX; ++s) v[s] = cmul(v[s], __ldg(Sy.td[0] + t + T * slot_q<NX, RX, 0>(s)));
             }
-            // the rows are read before the exchange (or, unstaged, the output) reuses them
-            if constexpr (Cfg::INPLACE || !UPDATE) __syncthreads();
+            __syncthreads();  // the rows are read before the exchange (or, unstaged, the output) reuses them
         }
-        fft_run<NX, RX, +1, true>(v, ex + (size_t)lu * SL, 1, t, tw, tc, RowSync<T>());
+        fft_run<NX, RX, +1, true>(v, row, 1, t, tw, tc, RowSync<T>());
         if constexpr (UPDATE) {
             // (the wait's barrier also ends every read of the exchange by the inverse transform)
             if (lost(1)) return;
             if (!yown) {
-                if (threadIdx.x == 0) {
-                    const uint32_t fb = (uint32_t)nrow * NX * sizeof(CT);
-                    fence_proxy_async_smem();  // the generic-proxy accesses of the buffer come before the copy's writes
-                    mbar_expect_tx(bar + 2, (pair ? 2u : 1u) * fb);
-                    bulk_g2s(ys, y + (long long)cs * d.N + v0, fb, bar + 2);
-                    if (pair) bulk_g2s(ys + H * NX, y + v0, fb, bar + 2);
-                }
+                fence_proxy_async_smem();  // the generic-proxy accesses of the buffer come before the copies' writes
+                y_in(bar + 2);
             }
             if (lost(2)) return;
         }
     } else if constexpr (HAS_B) {
         if (lost(0)) return;
     }
-    R s0 = (R)0, s1 = (R)0;
     if constexpr (UPDATE) {
+        R s0 = (R)0, s1 = (R)0;
         // the velocity's Pu (B x + y) in real space; the pressure has no such term
         const CT pu = pres ? mk<CT, R>((R)0, (R)0) : Sy.Pu;
+        CT* xo = x + fbase + t;
+        auto update = [&](auto is_pair) {
 #pragma unroll
-        for (int s = 0; s < RX; ++s) {
-            const int i0 = t + T * slot_q<NX, RX, np>(s);
-            const CT bv = B_at(i0);
-            const CT xv = xs[lu * NX + i0];
-            const CT wo = cfma(bv, xv, ys[lu * NX + i0]);
-            const CT z = cfma(pu, wo, v[s]);
-            const CT del = cmul(bv, cscale(csub(z, xv), nu));
-            const CT xn = cadd(xv, del);
-            if (valid) x[fbase + i0] = xn;
-            if constexpr (NORM) {
-                s0 += cabs2(del);
-                s1 += cabs2(xn);
+            for (int s = 0; s < RX; ++s) {
+                const int o = T * slot_q<NX, RX, np>(s);
+                const CT bv = B_at(o, is_pair);
+                const CT xv = xr[o], yv = yr[o];
+                const CT wo = cfma(bv, xv, yv);                 // B x + y
+                const CT zx = cfma(pu, wo, csub(v[s], xv));     // z - x
+                const CT bn = cscale(bv, nu);
+                const CT xn = cfma(bn, zx, xv);
+                if (valid) xo[o] = xn;
+                if constexpr (NORM) {
+                    s0 += cabs2(cmul(bn, zx));  // (not xn - x: that has lost x's low bits)
+                    s1 += cabs2(xn);
+                }
+                if constexpr (HAS_FWD) v[s] = cfma(bv, xn, yv);
             }
-            if constexpr (HAS_FWD) v[s] = cfma(bv, del, wo);  // B x + y of the updated x
-        }
+        };
+        if (pair) update(std::true_type());
+        else update(std::false_type());
         if constexpr (NORM) {
             if (!valid) { s0 = (R)0; s1 = (R)0; }
             block_sum2(s0, s1, partials + 2 * (long long)blockIdx.x);
@@ -435,27 +471,27 @@ k_rows(Dims d, Medium<R> M, Symbol<R> Sy, cplx<R>* __restrict__ x, const cplx<R>
     } else if constexpr (MODE == ROWS_FWD) {
 #pragma unroll
         for (int s = 0; s < RX; ++s) {
-            const int i0 = t + T * slot_q<NX, RX, 0>(s);
-            v[s] = cfma(B_at(i0), xs[lu * NX + i0], ys[lu * NX + i0]);
+            const int o = T * slot_q<NX, RX, 0>(s);
+            v[s] = cfma(pair ? B_at(o, std::true_type()) : B_at(o, std::false_type()), xr[o], yr[o]);
         }
     } else if constexpr (MODE == ROWS_COPY) {
 #pragma unroll
         for (int s = 0; s < RX; ++s) v[s] = x[fbase + t + T * slot_q<NX, RX, 0>(s)];
-    } else {  // ROWS_GREEN
+    } else {  // ROWS_GREEN (the 1 / N of the inverse transforms is in the symbol)
         const CT pu = pres ? mk<CT, R>((R)0, (R)0) : Sy.Pu;
         if (valid) {
 #pragma unroll
             for (int s = 0; s < RX; ++s) {
-                const int i0 = t + T * slot_q<NX, RX, np>(s);
-                // (the 1 / N of the inverse transforms is in the symbol, so v needs no further scaling)
-                w[fbase + i0] = cfma(pu, x[fbase + i0], v[s]);
+                const long long f = fbase + t + T * slot_q<NX, RX, np>(s);
+                w[f] = cfma(pu, x[f], v[s]);
             }
         }
     }
     if constexpr (HAS_FWD) {
-        fft_run<NX, RX, -1, true>(v, ex + (size_t)lu * SL, 1, t, tw, tc, RowSync<T>());
+        fft_run<NX, RX, -1, true>(v, row, 1, t, tw, tc, RowSync<T>());
+        CT* wo = w + fbase + t;
         if (pair) {  // q = p + tm_x u_x
-            CT* h = ex + (size_t)(isx ? lu : lu + H) * SL + t;
+            CT* h = ws + (isx ? lu : lu + H) * SL + t;
             __syncthreads();  // every exchange read is done
             if (isx) {
 #pragma unroll
@@ -464,10 +500,10 @@ k_rows(Dims d, Medium<R> M, Symbol<R> Sy, cplx<R>* __restrict__ x, const cplx<R>
             __syncthreads();
             if (isx || !valid) return;
 #pragma unroll
-            for (int s = 0; s < RX; ++s) w[fbase + t + T * slot_q<NX, RX, np>(s)] = cadd(v[s], h[s * T]);
+            for (int s = 0; s < RX; ++s) wo[T * slot_q<NX, RX, np>(s)] = cadd(v[s], h[s * T]);
         } else if (valid) {
 #pragma unroll
-            for (int s = 0; s < RX; ++s) w[fbase + t + T * slot_q<NX, RX, np>(s)] = v[s];
+            for (int s = 0; s < RX; ++s) wo[T * slot_q<NX, RX, np>(s)] = v[s];
         }
     }
 }

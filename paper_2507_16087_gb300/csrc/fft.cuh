@@ -162,14 +162,15 @@ template <int r, int S, typename CT> __host__ __device__ __forceinline__ void df
 }
 
 // ------------------------------------------------------------------- plans
-// Radix of the step that reduces `rem` (the part of N not yet transformed).
+// Radix of the step that reduces `rem` (the part of N not yet transformed); a factor of 3 comes last, so that the
+// strides of the earlier passes are powers of two.
 __host__ __device__ constexpr int plan_step(int rem, int R)
 {
-    return (rem % 3 == 0 && R % 3 == 0) ? 3
-         : (rem % 16 == 0 && R % 16 == 0) ? 16
+    return (rem % 16 == 0 && R % 16 == 0) ? 16
          : (rem % 8 == 0 && R % 8 == 0) ? 8
          : (rem % 4 == 0 && R % 4 == 0) ? 4
-         : (rem % 2 == 0 && R % 2 == 0) ? 2 : 0;
+         : (rem % 2 == 0 && R % 2 == 0) ? 2
+         : (rem % 3 == 0 && R % 3 == 0) ? 3 : 0;
 }
 __host__ __device__ constexpr int plan_radix(int N, int R, int p)
 {
@@ -289,19 +290,28 @@ __device__ __forceinline__ void pass_compute(CT (&v)[R], int tid, const CT* __re
     }
 }
 
-// Shared-memory address of element e.  Column tiles (PAD = false): e * ss.
-// A row stored contiguously (PAD = true): a swizzle that keeps the Stockham
-// writes (stride r) and reads (stride N/r) of a 16-lane phase on distinct
-// banks: XOR of bits 3..6 into bits 0..3 when N >= 128, else a skew.
-template <int N> __host__ __device__ constexpr int row_swizzle(int e)
-{
-    return (N >= 128 && N % 16 == 0) ? (e ^ ((e >> 3) & 15)) : (N == 64 ? e + (e >> 3) + (e >> 6) : e + (e >> 4));
-}
-template <int N, bool PAD> __device__ __forceinline__ int sm_addr(int e, int ss) { return PAD ? row_swizzle<N>(e) : e * ss; }
-template <int N, bool PAD> __host__ __device__ constexpr int sm_len()
-{
-    return PAD ? ((N >= 128 && N % 16 == 0) ? N : row_swizzle<N>(N - 1) + 1) : N;
-}
+// Exchange layout of a row (PAD): element e at e + e / 16 (8-byte values; e / 8 for 16-byte ones), so that the
+// Stockham writes (stride r) and reads (stride N/r) of the lanes that share a shared-memory phase fall on distinct
+// banks.  For power-of-two N the split pad(a + b) = pad(a) + pad(b) holds between a thread's own part of a position
+// and the compile-time part (no carry crosses a 16), so every access is one base register plus an immediate.  The
+// row pitch SL shifts consecutive rows by T places: the rows of one phase (T < 16 lanes each) don't collide either.
+template <typename CT, int N, int T> struct RowPad {
+    static constexpr int SH = sizeof(CT) == 8 ? 4 : 3;
+    __host__ __device__ static constexpr int pad(int e) { return e + (e >> SH); }
+    static constexpr int M = 1 << SH;
+    static constexpr int STEP = sizeof(CT) == 8 ? 2 : 1;  // rows start on 16-byte boundaries
+    __host__ __device__ static constexpr int pitch()
+    {
+        const int want = T < M ? (T < STEP ? STEP : T) : 0;
+        int sl = (pad(N - 1) + STEP) / STEP * STEP;
+        while (want != 0 && sl % M != want) sl += STEP;
+        return sl;
+    }
+    static constexpr int SL = pitch();
+    static constexpr bool LINEAR = (N & (N - 1)) == 0;
+    // position a (the thread's) + b (compile-time)
+    __host__ __device__ static constexpr int at(int a, int b) { return LINEAR ? pad(a) + pad(b) : pad(a + b); }
+};
 
 template <int N, int R, int T, int P, bool PAD, typename CT, typename Sync>
 __device__ __forceinline__ void pass_exchange(CT (&v)[R], CT* sm, int ss, int tid, Sync sync)
@@ -309,20 +319,21 @@ __device__ __forceinline__ void pass_exchange(CT (&v)[R], CT* sm, int ss, int ti
     constexpr int r = plan_radix(N, R, P);
     constexpr int NS = plan_ns(N, R, P);
     constexpr int rn = plan_radix(N, R, P + 1);
+    using L = RowPad<CT, N, T>;
     sync();
 #pragma unroll
     for (int m = 0; m < R / r; ++m) {
         const int j = tid + T * m;
         const int idx = (j / NS) * NS * r + (j % NS);
 #pragma unroll
-        for (int k = 0; k < r; ++k) sm[sm_addr<N, PAD>(idx + k * NS, ss)] = v[m * r + k];
+        for (int k = 0; k < r; ++k) sm[PAD ? L::at(idx, k * NS) : (idx + k * NS) * ss] = v[m * r + k];
     }
     sync();
 #pragma unroll
     for (int m = 0; m < R / rn; ++m) {
         const int j = tid + T * m;
 #pragma unroll
-        for (int k = 0; k < rn; ++k) v[m * rn + k] = sm[sm_addr<N, PAD>(j + k * (N / rn), ss)];
+        for (int k = 0; k < rn; ++k) v[m * rn + k] = sm[PAD ? L::at(j, k * (N / rn)) : (j + k * (N / rn)) * ss];
     }
 }
 
