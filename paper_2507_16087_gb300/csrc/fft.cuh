@@ -26,9 +26,26 @@ template <> struct real_of<float2> { using T = float; };
 template <> struct real_of<double2> { using T = double; };
 
 template <typename CT, typename R> __host__ __device__ __forceinline__ CT mk(R a, R b) { CT c; c.x = a; c.y = b; return c; }
-__host__ __device__ __forceinline__ float2 cadd(float2 a, float2 b) { return make_float2(a.x + b.x, a.y + b.y); }
+// float32 pairs: one packed instruction (f32x2) where both parts take the same operation, which is most of an FFT's
+// butterflies; the kernels are bound by issue, so halving those instructions is what counts (each part is rounded as
+// by the scalar instruction)
+__host__ __device__ __forceinline__ float2 cadd(float2 a, float2 b)
+{
+#if defined(__CUDA_ARCH__) && __CUDA_ARCH__ >= 1000
+    return __fadd2_rn(a, b);
+#else
+    return make_float2(a.x + b.x, a.y + b.y);
+#endif
+}
 __host__ __device__ __forceinline__ double2 cadd(double2 a, double2 b) { return make_double2(a.x + b.x, a.y + b.y); }
-__host__ __device__ __forceinline__ float2 csub(float2 a, float2 b) { return make_float2(a.x - b.x, a.y - b.y); }
+__host__ __device__ __forceinline__ float2 csub(float2 a, float2 b)
+{
+#if defined(__CUDA_ARCH__) && __CUDA_ARCH__ >= 1000
+    return __ffma2_rn(b, make_float2(-1.0f, -1.0f), a);
+#else
+    return make_float2(a.x - b.x, a.y - b.y);
+#endif
+}
 __host__ __device__ __forceinline__ double2 csub(double2 a, double2 b) { return make_double2(a.x - b.x, a.y - b.y); }
 __host__ __device__ __forceinline__ float2 cmul(float2 a, float2 b)
 {
@@ -47,7 +64,34 @@ __host__ __device__ __forceinline__ double2 cmulc(double2 a, double2 b)
 {
     return make_double2(fma(a.x, b.x, a.y * b.y), fma(a.y, b.x, -a.x * b.y));
 }
-__host__ __device__ __forceinline__ float2 cscale(float2 a, float s) { return make_float2(a.x * s, a.y * s); }
+__host__ __device__ __forceinline__ float2 cscale(float2 a, float s)
+{
+#if defined(__CUDA_ARCH__) && __CUDA_ARCH__ >= 1000
+    return __fmul2_rn(a, make_float2(s, s));
+#else
+    return make_float2(a.x * s, a.y * s);
+#endif
+}
+// a s + b with a real s
+__host__ __device__ __forceinline__ float2 caxpy(float2 a, float s, float2 b)
+{
+#if defined(__CUDA_ARCH__) && __CUDA_ARCH__ >= 1000
+    return __ffma2_rn(a, make_float2(s, s), b);
+#else
+    return make_float2(fmaf(a.x, s, b.x), fmaf(a.y, s, b.y));
+#endif
+}
+__host__ __device__ __forceinline__ double2 caxpy(double2 a, double s, double2 b)
+{
+    return make_double2(fma(a.x, s, b.x), fma(a.y, s, b.y));
+}
+// a + S i b
+template <int S, typename CT> __host__ __device__ __forceinline__ CT cadd_i(CT a, CT b)
+{
+    if constexpr (S > 0) { a.x -= b.y; a.y += b.x; }
+    else { a.x += b.y; a.y -= b.x; }
+    return a;
+}
 __host__ __device__ __forceinline__ double2 cscale(double2 a, double s) { return make_double2(a.x * s, a.y * s); }
 __host__ __device__ __forceinline__ float2 cconj(float2 a) { return make_float2(a.x, -a.y); }
 __host__ __device__ __forceinline__ double2 cconj(double2 a) { return make_double2(a.x, -a.y); }
@@ -69,11 +113,11 @@ template <int S, typename CT> __host__ __device__ __forceinline__ void dft2(CT* 
 template <int S, typename CT> __host__ __device__ __forceinline__ void dft4(CT* v)
 {
     CT s0 = cadd(v[0], v[2]), d0 = csub(v[0], v[2]);
-    CT s1 = cadd(v[1], v[3]), d1 = mul_si<S>(csub(v[1], v[3]));
+    CT s1 = cadd(v[1], v[3]), d1 = csub(v[1], v[3]);
     v[0] = cadd(s0, s1);
     v[2] = csub(s0, s1);
-    v[1] = cadd(d0, d1);
-    v[3] = csub(d0, d1);
+    v[1] = cadd_i<S>(d0, d1);
+    v[3] = cadd_i<-S>(d0, d1);
 }
 
 template <int S, typename CT> __host__ __device__ __forceinline__ void dft3(CT* v)
@@ -81,13 +125,11 @@ template <int S, typename CT> __host__ __device__ __forceinline__ void dft3(CT* 
     using R = typename real_of<CT>::T;
     const R h = (R)0.86602540378443864676372317075294;  // sin(2 pi / 3)
     CT t = cadd(v[1], v[2]);
-    CT u = csub(v[1], v[2]);
-    CT a = v[0];
-    CT m = mk<CT, R>(a.x - (R)0.5 * t.x, a.y - (R)0.5 * t.y);
-    CT iu = mul_si<S>(cscale(u, h));
-    v[0] = cadd(a, t);
-    v[1] = cadd(m, iu);
-    v[2] = csub(m, iu);
+    CT u = cscale(csub(v[1], v[2]), h);
+    CT m = caxpy(t, (R)-0.5, v[0]);
+    v[0] = cadd(v[0], t);
+    v[1] = cadd_i<S>(m, u);
+    v[2] = cadd_i<-S>(m, u);
 }
 
 // 8 = 2 x 4: even/odd 4-point DFTs combined with w8^q = exp(S 2 pi i q / 8)
@@ -99,18 +141,17 @@ template <int S, typename CT> __host__ __device__ __forceinline__ void dft8(CT* 
     CT o[4] = {v[1], v[3], v[5], v[7]};
     dft4<S>(e);
     dft4<S>(o);
-    // w8^1 = c (1 + S i), w8^2 = S i, w8^3 = c (-1 + S i)
-    CT o1 = mk<CT, R>(c * (o[1].x - (R)S * o[1].y), c * (o[1].y + (R)S * o[1].x));
-    CT o2 = mul_si<S>(o[2]);
-    CT o3 = mk<CT, R>(c * (-o[3].x - (R)S * o[3].y), c * (-o[3].y + (R)S * o[3].x));
+    // w8^1 = c (1 + S i), w8^2 = S i, w8^3 = -c (1 - S i); the scaling rides on the combining additions
+    const CT o1 = cadd_i<S>(o[1], o[1]);
+    const CT o3 = cadd_i<-S>(o[3], o[3]);
     v[0] = cadd(e[0], o[0]);
     v[4] = csub(e[0], o[0]);
-    v[1] = cadd(e[1], o1);
-    v[5] = csub(e[1], o1);
-    v[2] = cadd(e[2], o2);
-    v[6] = csub(e[2], o2);
-    v[3] = cadd(e[3], o3);
-    v[7] = csub(e[3], o3);
+    v[1] = caxpy(o1, c, e[1]);
+    v[5] = caxpy(o1, -c, e[1]);
+    v[2] = cadd_i<S>(e[2], o[2]);
+    v[6] = cadd_i<-S>(e[2], o[2]);
+    v[3] = caxpy(o3, -c, e[3]);
+    v[7] = caxpy(o3, c, e[3]);
 }
 
 // 16 = 4 x 4: n = 4 n1 + n2, k = k1 + 4 k2; inner 4-point DFTs over n1, twiddles
@@ -130,23 +171,29 @@ template <int S, typename CT> __host__ __device__ __forceinline__ void dft16(CT*
         for (int k1 = 0; k1 < 4; ++k1) a[n2][k1] = t[k1];
     }
     const CT w1 = mk<CT, R>(c1, (R)S * s1);
-    const CT w2 = mk<CT, R>(h, (R)S * h);
     const CT w3 = mk<CT, R>(s1, (R)S * c1);
-    const CT w6 = mk<CT, R>(-h, (R)S * h);
     const CT w9 = mk<CT, R>(-c1, -(R)S * s1);
     a[1][1] = cmul(a[1][1], w1);
-    a[1][2] = cmul(a[1][2], w2);
+    a[1][2] = cscale(cadd_i<S>(a[1][2], a[1][2]), h);     // w2 = h (1 + S i)
     a[1][3] = cmul(a[1][3], w3);
-    a[2][1] = cmul(a[2][1], w2);
-    a[2][2] = mul_si<S>(a[2][2]);
-    a[2][3] = cmul(a[2][3], w6);
+    a[2][1] = cscale(cadd_i<S>(a[2][1], a[2][1]), h);
+    a[2][3] = cscale(cadd_i<-S>(a[2][3], a[2][3]), -h);   // w6 = -h (1 - S i)
     a[3][1] = cmul(a[3][1], w3);
-    a[3][2] = cmul(a[3][2], w6);
+    a[3][2] = cscale(cadd_i<-S>(a[3][2], a[3][2]), -h);
     a[3][3] = cmul(a[3][3], w9);
 #pragma unroll
     for (int k1 = 0; k1 < 4; ++k1) {
         CT t[4] = {a[0][k1], a[1][k1], a[2][k1], a[3][k1]};
-        dft4<S>(t);
+        if (k1 != 2) {
+            dft4<S>(t);
+        } else {  // w4 = S i on t[2] rides on the first butterflies
+            const CT s0 = cadd_i<S>(t[0], t[2]), d0 = cadd_i<-S>(t[0], t[2]);
+            const CT s2 = cadd(t[1], t[3]), d2 = csub(t[1], t[3]);
+            t[0] = cadd(s0, s2);
+            t[2] = csub(s0, s2);
+            t[1] = cadd_i<S>(d0, d2);
+            t[3] = cadd_i<-S>(d0, d2);
+        }
 #pragma unroll
         for (int k2 = 0; k2 < 4; ++k2) v[k1 + 4 * k2] = t[k2];
     }
