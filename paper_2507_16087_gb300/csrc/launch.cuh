@@ -16,7 +16,8 @@ template <typename R> __host__ __device__ constexpr int r_rows(int n)
 {
     return (n % 3 == 0) ? ((sizeof(R) == 4 && n >= 192) ? 24 : 12) : ((sizeof(R) == 4 && n >= 128) ? 16 : 8);
 }
-// strided axes (two transforms a thread): 16 values for float32 axes of 128 and more points, else 8; 3*2^k: 12
+// strided axes (two transforms a thread): 16 values for float32 axes of 128 and more points, else 8; 3*2^k: 12 (8 values
+// at 128^3 / 256^3 / 512^3: last axis 24.2 / 161 / 1581 us against 22.1 / 137 / 1471)
 template <typename R> __host__ __device__ constexpr int r_axis(int n)
 {
     return (n % 3 == 0) ? 12 : ((sizeof(R) == 4 && n >= 128) ? 16 : 8);
@@ -26,11 +27,13 @@ template <typename R> __host__ __device__ constexpr int r_last(int n, int = 2) {
 template <typename R> __host__ __device__ constexpr int r_tile(int n) { return (n % 3 == 0) ? 12 : 8; }
 
 __host__ __device__ constexpr int max_i(int a, int b) { return a > b ? a : b; }
-// columns of a tile: whole 128-byte lines where a tile of two transforms leaves room for several blocks an SM
+// columns of a tile: whole 128-byte lines where a tile of two transforms leaves room for several blocks an SM (us of
+// the last axis, columns: 128^3 24.2 / 22.1 / 25.4 with 8 / 16 / 32, 256^3 149 / 137 with 8 / 16, 512^3 2261 / 1471 /
+// 1622 with 4 / 8 / 16, 1024^2 23.0 / 27.5 with 4 / 8, 2048^2 112 / 90 with 2 / 4)
 template <typename R> __host__ __device__ constexpr int cols_big(int n)
 {
     const int t = n / r_axis<R>(n);
-    return sizeof(R) == 4 ? max_i(n <= 256 ? 16 : (n <= 1024 ? 8 : 4), 128 / t)
+    return sizeof(R) == 4 ? max_i(n <= 256 ? 16 : (n <= 512 ? 8 : 4), 128 / t)
                           : max_i(n <= 128 ? 8 : (n <= 512 ? 4 : 2), 64 / t);
 }
 // small grids: 32-byte rows, as many blocks as that gives
@@ -63,7 +66,25 @@ template <typename R> struct Plan {
     int* err = nullptr;    // device error word of the staged copies' bounded waits
 };
 
-constexpr int kWaveBlocks = 2 * 152;  // two blocks on every SM
+// One launch; `dependent`: the kernel may be scheduled while the one before it in the stream still runs (it waits in
+// grid_wait).  Only for kernels whose predecessor is one of the kernels here.
+template <typename Kern, typename... Args>
+cudaError_t launch(Kern kern, long long grid, int threads, size_t smem, cudaStream_t st, bool dependent, Args... args)
+{
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = dim3((unsigned)grid);
+    cfg.blockDim = dim3((unsigned)threads);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = st;
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = at;
+    cfg.numAttrs = dependent ? 1 : 0;
+    return cudaLaunchKernelEx(&cfg, kern, args...);
+}
+
+constexpr int kWaveBlocks = 2 * kSMs;  // two blocks on every SM
 
 // transform units (x rows of one component) of a row block: as many as 64 threads hold, halved while the grid
 // would leave SMs without two blocks
@@ -119,9 +140,9 @@ cudaError_t rows_nm(const Plan<R>& P, cplx<R>* x, const cplx<R>* y, cplx<R>* w, 
     // a grid of few blocks an SM gives y a buffer of its own, its copy in flight from the start (64^3: 12.3 against
     // 14.1 us; above that the room costs more blocks than the wait does time: 192^3 331 against 296 us)
     const int ysep = g.blocks <= 4 * kWaveBlocks && Cfg::smem(g.units, true) < kMaxDynSmem ? 1 : 0;
-    kern<<<g.blocks, g.units * Cfg::T, Cfg::smem(g.units, ysep != 0), st>>>(
-        P.d, P.M, P.Sy[adj ? 1 : 0], x, y, w, P.tw[0], g.npair, g.nsingle, ysep, adj, nu, partials, P.err);
-    return cudaGetLastError();
+    // the modes that start a chain follow other work (x and y may have just been written)
+    return launch(kern, g.blocks, g.units * Cfg::T, Cfg::smem(g.units, ysep != 0), st, MODE != ROWS_FWD && MODE != ROWS_COPY,
+                  P.d, P.M, P.Sy[adj ? 1 : 0], x, y, w, P.tw[0], g.npair, g.nsingle, ysep, adj, nu, partials, P.err);
 }
 
 template <typename R, int N>
@@ -163,9 +184,8 @@ cudaError_t rows_op_n(const Plan<R>& P, const cplx<R>* x, const cplx<R>* y, cplx
     static const cudaError_t attr = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, kMax);
     if (attr != cudaSuccess) return attr;
     const RowGrid g = row_grid<R, N>(P.d);
-    kern<<<g.blocks, g.units * Cfg::T, (size_t)g.units * Cfg::SL * sizeof(cplx<R>), st>>>(
-        P.d, P.M, P.L[adj ? 1 : 0], x, y, w, P.tw[0], g.npair, g.nsingle, mode, adj, partials);
-    return cudaGetLastError();
+    return launch(kern, g.blocks, g.units * Cfg::T, (size_t)g.units * Cfg::SL * sizeof(cplx<R>), st, true, P.d, P.M,
+                  P.L[adj ? 1 : 0], x, y, w, P.tw[0], g.npair, g.nsingle, mode, adj, partials);
 }
 
 // x axis and diagonal of the operator (after launch_deriv of the other axes)
@@ -181,8 +201,9 @@ cudaError_t launch_rows_op(const Plan<R>& P, const cplx<R>* x, const cplx<R>* y,
     }
 }
 
-// true when `columns` columns in tiles of `cols` leave SMs without two blocks: the launch takes the small tiles
-inline bool small_tiles(long long columns, int cols) { return (columns + cols - 1) / cols < kWaveBlocks; }
+// true when `columns` columns in tiles of `cols` leave SMs without a block: the launch takes the small tiles (64^3, 256
+// tiles: 20.3 us an iteration with the big ones against 20.9; 512^2, 64 tiles: 17.8 against 15.9)
+inline bool small_tiles(long long columns, int cols) { return (columns + cols - 1) / cols < kSMs; }
 
 template <typename R, int N, int RA, int COLS, int S> cudaError_t axis2_tile(const Plan<R>& P, cplx<R>* w, int adj, cudaStream_t st)
 {
@@ -193,8 +214,7 @@ template <typename R, int N, int RA, int COLS, int S> cudaError_t axis2_tile(con
     const int ncol = P.d.n0 * P.d.n2;
     const int npair = (ncol + COLS - 1) / COLS, nz = (ncol / 2 + COLS - 1) / COLS;
     const Symbol<R>& Sy = P.Sy[adj ? 1 : 0];
-    kern<<<npair + nz, Cfg::THREADS, Cfg::SMEM, st>>>(P.d, w, P.tw[1], S < 0 ? Sy.tm[1] : Sy.td[1], npair);
-    return cudaGetLastError();
+    return launch(kern, npair + nz, Cfg::THREADS, Cfg::SMEM, st, true, P.d, w, P.tw[1], S < 0 ? Sy.tm[1] : Sy.td[1], npair);
 }
 template <typename R, int N, int S> cudaError_t axis2_n(const Plan<R>& P, cplx<R>* w, int adj, cudaStream_t st)
 {
@@ -224,8 +244,7 @@ template <typename R, int N, int RL, int COLS> cudaError_t last2_tile(const Plan
     static const cudaError_t attr = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)Cfg::SMEM);
     if (attr != cudaSuccess) return attr;
     const long long ncol = P.d.D == 3 ? (long long)P.d.n0 * P.d.n1 : P.d.n0;
-    kern<<<(unsigned)((ncol + COLS - 1) / COLS), Cfg::THREADS, Cfg::SMEM, st>>>(P.d, P.Sy[adj ? 1 : 0], w, P.tw[P.d.D - 1]);
-    return cudaGetLastError();
+    return launch(kern, (ncol + COLS - 1) / COLS, Cfg::THREADS, Cfg::SMEM, st, true, P.d, P.Sy[adj ? 1 : 0], w, P.tw[P.d.D - 1]);
 }
 template <typename R, int N> cudaError_t last2_n(const Plan<R>& P, cplx<R>* w, int adj, cudaStream_t st)
 {
@@ -257,8 +276,8 @@ cudaError_t deriv_tile(const Plan<R>& P, const cplx<R>* x, cplx<R>* w, int e, in
     if (attr != cudaSuccess) return attr;
     const int n[3] = {P.d.n0, P.d.n1, P.d.n2};
     const long long ncol = P.d.N / n[e];
-    kern<<<(unsigned)((ncol + COLS - 1) / COLS), Cfg::THREADS, Cfg::SMEM, st>>>(P.d, P.L[adj ? 1 : 0], x, w, P.tw[e], e, add);
-    return cudaGetLastError();
+    return launch(kern, (ncol + COLS - 1) / COLS, Cfg::THREADS, Cfg::SMEM, st, add != 0, P.d, P.L[adj ? 1 : 0], x, w, P.tw[e],
+                  e, add);
 }
 template <typename R, int N>
 cudaError_t deriv_n(const Plan<R>& P, const cplx<R>* x, cplx<R>* w, int e, int add, int adj, cudaStream_t st)
