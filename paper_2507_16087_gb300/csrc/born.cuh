@@ -144,16 +144,18 @@ __device__ __forceinline__ cplx<R> born_B(const Medium<R>& M, const RowB<R>& rb,
 // the one before it is complete and visible; only what the direct predecessor writes has to wait.
 // The trigger comes before a block's last stores: the next kernel's blocks then find free SMs and start evenly.  Given
 // right after the wait it packs them onto the SMs that finish first (64^3 23.6 against 20.9 us an iteration, 512^2 19.3
-// against 15.7, 512^3 8.7 against 7.5 ms); only a grid of at most one block an SM gains (128^2 8.1 against 9.4 us).
+// against 15.7, 512^3 8.7 against 7.5 ms); only a float32 grid of at most one block an SM gains (128^2 8.1 against 9.4
+// us; float64 kernels are not launched this way, see kDependent in launch.cuh).
 __device__ __forceinline__ void grid_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void grid_trigger() { asm volatile("griddepcontrol.launch_dependents;"); }
 constexpr int kSMs = 152;
-__device__ __forceinline__ void grid_trigger_small()  // (predicated: a branch here splits the loads that follow)
+template <typename R> __device__ __forceinline__ void grid_trigger_small()  // (predicated: a branch here splits the loads that follow)
 {
-    asm volatile(
-        "{\n\t.reg .pred p;\n\t"
-        "setp.le.u32 p, %0, %1;\n\t"
-        "@p griddepcontrol.launch_dependents;\n\t}" ::"r"(gridDim.x), "n"(kSMs));
+    if constexpr (sizeof(R) == 4)
+        asm volatile(
+            "{\n\t.reg .pred p;\n\t"
+            "setp.le.u32 p, %0, %1;\n\t"
+            "@p griddepcontrol.launch_dependents;\n\t}" ::"r"(gridDim.x), "n"(kSMs));
 }
 
 template <int T> struct RowSync {
@@ -365,7 +367,7 @@ k_rows(Dims d, Medium<R> M, Symbol<R> Sy, cplx<R>* __restrict__ x, const cplx<R>
     // w goes first, the transform waits for nothing else (512^3 3.54 against 3.64 ms, 2048^2 154 against 161 us).
     auto w_in = [&]() {
         grid_wait();
-        grid_trigger_small();
+        grid_trigger_small<R>();
         if constexpr (UPDATE) rows_in(ws, w + (long long)cs * d.N + v0, SL, FB, bar);
     };
     auto y_in = [&](uint64_t* on) {
@@ -598,7 +600,7 @@ k_axis2(Dims d, cplx<R>* __restrict__ w, const cplx<R>* __restrict__ tw, const c
     const long long st = (long long)T * d.n0;
     CT v[2][RA];
     grid_wait();
-    grid_trigger_small();
+    grid_trigger_small<R>();
     col_load<NA, RA, 0>(v[0], a, st);
     if (S < 0 || !pair) {
         col_load<NA, RA, 0>(v[1], b, st);
@@ -639,7 +641,7 @@ k_last2(Dims d, Symbol<R> Sy, cplx<R>* __restrict__ w, const cplx<R>* __restrict
     const long long st = (long long)T * ncol;
     CT v[2][RL];
     grid_wait();
-    if (gridDim.x <= kSMs) grid_trigger();  // (a branch, not the predicated form: 137 against 151 us at 256^3)
+    if (sizeof(R) == 4 && gridDim.x <= kSMs) grid_trigger();  // (a branch, not the predicated form: 137 against 151 us at 256^3)
     col_load<NL, RL, 0>(v[0], a, st);
     col_load<NL, RL, 0>(v[1], b, st);
     R k2c = Sy.c3.x;
@@ -696,7 +698,7 @@ k_deriv2(Dims d, LOp<R> L, const cplx<R>* __restrict__ x, cplx<R>* __restrict__ 
     const long long st = (long long)T * astride;
     CT v[2][RA];
     grid_wait();
-    grid_trigger_small();
+    grid_trigger_small<R>();
     col_load<N, RA, 0>(v[0], x + oa, st);
     col_load<N, RA, 0>(v[1], x + ob, st);
     fft_run_multi<N, RA, 2, -1, 0, true>(v, sm + col, COLS, N * COLS, t, tw, BlockSync());
@@ -765,7 +767,7 @@ k_rows_op(Dims d, Medium<R> M, LOp<R> L, const cplx<R>* __restrict__ x, const cp
     const CT la = pres ? L.la2 : L.la1;
     CT v[RX];
     grid_wait();
-    grid_trigger_small();
+    grid_trigger_small<R>();
     if (pair) {
         TwCache<NX, RX, CT> tc;
         tw_load<NX, RX, T>(tc, t, tw);

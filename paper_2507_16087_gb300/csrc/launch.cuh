@@ -23,8 +23,14 @@ template <typename R> __host__ __device__ constexpr int r_axis(int n)
     return (n % 3 == 0) ? 12 : ((sizeof(R) == 4 && n >= 128) ? 16 : 8);
 }
 template <typename R> __host__ __device__ constexpr int r_last(int n, int = 2) { return r_axis<R>(n); }
-// small grids (see small_tiles): 8 values a thread at every 2^k extent, so that a column has more threads
-template <typename R> __host__ __device__ constexpr int r_tile(int n) { return (n % 3 == 0) ? 12 : 8; }
+// small grids: fewer values a thread, so that a transform has more threads.  float32 (see small_tiles): 8 at every 2^k
+// extent.  float64 (see few_warps): 4, and 6 up to 48 points: an SM sub-partition issues one FP64 warp instruction in
+// 64 cycles, so a grid of fewer warps than there are sub-partitions takes as long as one warp's instructions.
+template <typename R> __host__ __device__ constexpr int r_tile(int n)
+{
+    return sizeof(R) == 4 ? ((n % 3 == 0) ? 12 : 8) : ((n % 3 == 0) ? (n <= 48 ? 6 : 12) : (n <= 512 ? 4 : 8));
+}
+template <typename R> __host__ __device__ constexpr int r_rows_tile(int n) { return sizeof(R) == 4 ? r_rows<R>(n) : r_tile<R>(n); }
 
 __host__ __device__ constexpr int max_i(int a, int b) { return a > b ? a : b; }
 // columns of a tile: whole 128-byte lines where a tile of two transforms leaves room for several blocks an SM (us of
@@ -34,13 +40,15 @@ template <typename R> __host__ __device__ constexpr int cols_big(int n)
 {
     const int t = n / r_axis<R>(n);
     return sizeof(R) == 4 ? max_i(n <= 256 ? 16 : (n <= 512 ? 8 : 4), 128 / t)
-                          : max_i(n <= 128 ? 8 : (n <= 512 ? 4 : 2), 64 / t);
+                          // float64 is bound by the FP64 pipes: small blocks, spread evenly (64^3: last axis 52.7 us
+                          // with 4 columns, 58.7 with 8; 1024^2 312 with 1, 359 with 2; 2048^2 1407 and 1335)
+                          : max_i(n == 1024 ? 1 : 2, 32 / t);
 }
-// small grids: 32-byte rows, as many blocks as that gives
+// small grids: 32-byte rows (float64 16), as many blocks as that gives
 template <typename R> __host__ __device__ constexpr int cols_small(int n)
 {
     const int t = n / r_tile<R>(n);
-    return max_i(sizeof(R) == 4 ? 4 : 2, 32 / t);
+    return max_i(sizeof(R) == 4 ? 4 : 1, 32 / t);
 }
 
 #define CBS_FOR_EACH_SIZE(X) X(8) X(12) X(16) X(24) X(32) X(48) X(64) X(96) X(128) X(192) X(256) X(512) X(1024) X(2048)
@@ -84,17 +92,32 @@ cudaError_t launch(Kern kern, long long grid, int threads, size_t smem, cudaStre
     return cudaLaunchKernelEx(&cfg, kern, args...);
 }
 
+// float32 only: float64 blocks, bound by their SM's FP64 pipe, gain 1-4 % on small grids but 25 % is lost where the next
+// kernel's blocks are packed onto the SMs that finish first (256^2: 73.5 against 58.7 us an iteration)
+template <typename R> constexpr bool kDependent = sizeof(R) == 4;
+
 constexpr int kWaveBlocks = 2 * kSMs;  // two blocks on every SM
+
+// float64 grids whose threads, each with r values, make fewer warps than there are SM sub-partitions (4 an SM)
+template <typename R> inline bool few_warps(long long values, int r)
+{
+    return sizeof(R) == 8 && values / r < 32LL * 4 * kSMs;
+}
 
 // transform units (x rows of one component) of a row block: as many as 64 threads hold, halved while the grid
 // would leave SMs without two blocks
-template <typename R, int N> inline int rows_units_n(const Dims& d)
+template <typename R, int N, int RX> inline int rows_units_n(const Dims& d)
 {
-    using Cfg = RowCfg<R, N, r_rows<R>(N)>;
+    using Cfg = RowCfg<R, N, RX>;
     const long long units = (long long)(d.D + 1) * (d.N / N);
     int u = Cfg::UMAX;
     while (u > Cfg::UMIN && units / u < kWaveBlocks) u /= 2;
     return u;
+}
+// values a thread of the row kernels on this grid: r_rows, or r_rows_tile when that leaves too few warps
+template <typename R, int N> inline bool rows_tiny(const Dims& d)
+{
+    return r_rows_tile<R>(N) < r_rows<R>(N) && few_warps<R>((long long)(d.D + 1) * d.N, r_rows<R>(N));
 }
 
 struct RowGrid {
@@ -103,7 +126,7 @@ struct RowGrid {
 template <typename R, int N> inline RowGrid row_grid(const Dims& d)
 {
     RowGrid g;
-    g.units = rows_units_n<R, N>(d);
+    g.units = rows_tiny<R, N>(d) ? rows_units_n<R, N, r_rows_tile<R>(N)>(d) : rows_units_n<R, N, r_rows<R>(N)>(d);
     const long long rpc = d.N / N;
     g.npair = (int)((rpc + g.units / 2 - 1) / (g.units / 2));
     g.nsingle = (int)((rpc + g.units - 1) / g.units);
@@ -124,11 +147,10 @@ template <typename R> inline int rows_blocks(const Plan<R>& P)
 
 constexpr size_t kMaxDynSmem = 226 * 1024;  // 227 KiB less the reduction scratch
 
-template <typename R, int N, int MODE>
+template <typename R, int N, int RX, int MODE>
 cudaError_t rows_nm(const Plan<R>& P, cplx<R>* x, const cplx<R>* y, cplx<R>* w, int adj, R nu, double* partials,
                     cudaStream_t st)
 {
-    constexpr int RX = r_rows<R>(N);
     using Cfg = RowCfg<R, N, RX>;
     auto kern = k_rows<R, N, RX, MODE>;
     // once per process, thread-safe (function-local static)
@@ -141,23 +163,33 @@ cudaError_t rows_nm(const Plan<R>& P, cplx<R>* x, const cplx<R>* y, cplx<R>* w, 
     // 14.1 us; above that the room costs more blocks than the wait does time: 192^3 331 against 296 us)
     const int ysep = g.blocks <= 4 * kWaveBlocks && Cfg::smem(g.units, true) < kMaxDynSmem ? 1 : 0;
     // the modes that start a chain follow other work (x and y may have just been written)
-    return launch(kern, g.blocks, g.units * Cfg::T, Cfg::smem(g.units, ysep != 0), st, MODE != ROWS_FWD && MODE != ROWS_COPY,
-                  P.d, P.M, P.Sy[adj ? 1 : 0], x, y, w, P.tw[0], g.npair, g.nsingle, ysep, adj, nu, partials, P.err);
+    return launch(kern, g.blocks, g.units * Cfg::T, Cfg::smem(g.units, ysep != 0), st,
+                  kDependent<R> && MODE != ROWS_FWD && MODE != ROWS_COPY, P.d, P.M, P.Sy[adj ? 1 : 0], x, y, w, P.tw[0], g.npair, g.nsingle, ysep, adj, nu, partials, P.err);
+}
+
+template <typename R, int N, int RX>
+cudaError_t rows_rx(const Plan<R>& P, cplx<R>* x, const cplx<R>* y, cplx<R>* w, int mode, int adj, R nu,
+                    double* partials, cudaStream_t st)
+{
+    switch (mode) {
+    case ROWS_FWD: return rows_nm<R, N, RX, ROWS_FWD>(P, x, y, w, adj, nu, partials, st);
+    case ROWS_FUSED: return rows_nm<R, N, RX, ROWS_FUSED>(P, x, y, w, adj, nu, partials, st);
+    case ROWS_FUSED_NORM: return rows_nm<R, N, RX, ROWS_FUSED_NORM>(P, x, y, w, adj, nu, partials, st);
+    case ROWS_INV: return rows_nm<R, N, RX, ROWS_INV>(P, x, y, w, adj, nu, partials, st);
+    case ROWS_COPY: return rows_nm<R, N, RX, ROWS_COPY>(P, x, y, w, adj, nu, partials, st);
+    case ROWS_GREEN: return rows_nm<R, N, RX, ROWS_GREEN>(P, x, y, w, adj, nu, partials, st);
+    default: return cudaErrorInvalidValue;
+    }
 }
 
 template <typename R, int N>
 cudaError_t rows_n(const Plan<R>& P, cplx<R>* x, const cplx<R>* y, cplx<R>* w, int mode, int adj, R nu,
                    double* partials, cudaStream_t st)
 {
-    switch (mode) {
-    case ROWS_FWD: return rows_nm<R, N, ROWS_FWD>(P, x, y, w, adj, nu, partials, st);
-    case ROWS_FUSED: return rows_nm<R, N, ROWS_FUSED>(P, x, y, w, adj, nu, partials, st);
-    case ROWS_FUSED_NORM: return rows_nm<R, N, ROWS_FUSED_NORM>(P, x, y, w, adj, nu, partials, st);
-    case ROWS_INV: return rows_nm<R, N, ROWS_INV>(P, x, y, w, adj, nu, partials, st);
-    case ROWS_COPY: return rows_nm<R, N, ROWS_COPY>(P, x, y, w, adj, nu, partials, st);
-    case ROWS_GREEN: return rows_nm<R, N, ROWS_GREEN>(P, x, y, w, adj, nu, partials, st);
-    default: return cudaErrorInvalidValue;
+    if constexpr (r_rows_tile<R>(N) < r_rows<R>(N)) {
+        if (rows_tiny<R, N>(P.d)) return rows_rx<R, N, r_rows_tile<R>(N)>(P, x, y, w, mode, adj, nu, partials, st);
     }
+    return rows_rx<R, N, r_rows<R>(N)>(P, x, y, w, mode, adj, nu, partials, st);
 }
 
 // row kernels (see RowsMode); ROWS_COPY and ROWS_GREEN only read x
@@ -173,19 +205,28 @@ cudaError_t launch_rows(const Plan<R>& P, cplx<R>* x, const cplx<R>* y, cplx<R>*
     }
 }
 
-template <typename R, int N>
-cudaError_t rows_op_n(const Plan<R>& P, const cplx<R>* x, const cplx<R>* y, cplx<R>* w, int mode, int adj,
-                      double* partials, cudaStream_t st)
+template <typename R, int N, int RX>
+cudaError_t rows_op_rx(const Plan<R>& P, const cplx<R>* x, const cplx<R>* y, cplx<R>* w, int mode, int adj,
+                       double* partials, cudaStream_t st)
 {
-    constexpr int RX = r_rows<R>(N);
     using Cfg = RowCfg<R, N, RX>;
     auto kern = k_rows_op<R, N, RX>;
     constexpr int kMax = (int)((size_t)Cfg::UMAX * Cfg::SL * sizeof(cplx<R>));
     static const cudaError_t attr = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, kMax);
     if (attr != cudaSuccess) return attr;
     const RowGrid g = row_grid<R, N>(P.d);
-    return launch(kern, g.blocks, g.units * Cfg::T, (size_t)g.units * Cfg::SL * sizeof(cplx<R>), st, true, P.d, P.M,
+    return launch(kern, g.blocks, g.units * Cfg::T, (size_t)g.units * Cfg::SL * sizeof(cplx<R>), st, kDependent<R>, P.d, P.M,
                   P.L[adj ? 1 : 0], x, y, w, P.tw[0], g.npair, g.nsingle, mode, adj, partials);
+}
+
+template <typename R, int N>
+cudaError_t rows_op_n(const Plan<R>& P, const cplx<R>* x, const cplx<R>* y, cplx<R>* w, int mode, int adj,
+                      double* partials, cudaStream_t st)
+{
+    if constexpr (r_rows_tile<R>(N) < r_rows<R>(N)) {
+        if (rows_tiny<R, N>(P.d)) return rows_op_rx<R, N, r_rows_tile<R>(N)>(P, x, y, w, mode, adj, partials, st);
+    }
+    return rows_op_rx<R, N, r_rows<R>(N)>(P, x, y, w, mode, adj, partials, st);
 }
 
 // x axis and diagonal of the operator (after launch_deriv of the other axes)
@@ -201,9 +242,14 @@ cudaError_t launch_rows_op(const Plan<R>& P, const cplx<R>* x, const cplx<R>* y,
     }
 }
 
-// true when `columns` columns in tiles of `cols` leave SMs without a block: the launch takes the small tiles (64^3, 256
-// tiles: 20.3 us an iteration with the big ones against 20.9; 512^2, 64 tiles: 17.8 against 15.9)
-inline bool small_tiles(long long columns, int cols) { return (columns + cols - 1) / cols < kSMs; }
+// whether a strided axis of N points and `columns` columns (of two transforms) takes the small tiles: float32 when the
+// big ones leave SMs without a block (64^3, 256 tiles: 20.3 us an iteration with the big ones against 20.9; 512^2, 64
+// tiles: 17.8 against 15.9), float64 when the big ones make too few warps
+template <typename R, int N> inline bool small_tiles(long long columns)
+{
+    if (sizeof(R) == 8) return few_warps<R>(columns * N, r_axis<R>(N));
+    return (columns + cols_big<R>(N) - 1) / cols_big<R>(N) < kSMs;
+}
 
 template <typename R, int N, int RA, int COLS, int S> cudaError_t axis2_tile(const Plan<R>& P, cplx<R>* w, int adj, cudaStream_t st)
 {
@@ -214,13 +260,13 @@ template <typename R, int N, int RA, int COLS, int S> cudaError_t axis2_tile(con
     const int ncol = P.d.n0 * P.d.n2;
     const int npair = (ncol + COLS - 1) / COLS, nz = (ncol / 2 + COLS - 1) / COLS;
     const Symbol<R>& Sy = P.Sy[adj ? 1 : 0];
-    return launch(kern, npair + nz, Cfg::THREADS, Cfg::SMEM, st, true, P.d, w, P.tw[1], S < 0 ? Sy.tm[1] : Sy.td[1], npair);
+    return launch(kern, npair + nz, Cfg::THREADS, Cfg::SMEM, st, kDependent<R>, P.d, w, P.tw[1], S < 0 ? Sy.tm[1] : Sy.td[1], npair);
 }
 template <typename R, int N, int S> cudaError_t axis2_n(const Plan<R>& P, cplx<R>* w, int adj, cudaStream_t st)
 {
     constexpr int CB = cols_big<R>(N), CS = cols_small<R>(N);
-    if constexpr (CS < CB) {
-        if (small_tiles((long long)P.d.n0 * P.d.n2 * 3 / 2, CB))
+    if constexpr (CS != CB || r_tile<R>(N) != r_axis<R>(N)) {
+        if (small_tiles<R, N>((long long)P.d.n0 * P.d.n2 * 3 / 2))
             return axis2_tile<R, N, r_tile<R>(N), CS, S>(P, w, adj, st);
     }
     return axis2_tile<R, N, r_axis<R>(N), CB, S>(P, w, adj, st);
@@ -244,14 +290,14 @@ template <typename R, int N, int RL, int COLS> cudaError_t last2_tile(const Plan
     static const cudaError_t attr = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)Cfg::SMEM);
     if (attr != cudaSuccess) return attr;
     const long long ncol = P.d.D == 3 ? (long long)P.d.n0 * P.d.n1 : P.d.n0;
-    return launch(kern, (ncol + COLS - 1) / COLS, Cfg::THREADS, Cfg::SMEM, st, true, P.d, P.Sy[adj ? 1 : 0], w, P.tw[P.d.D - 1]);
+    return launch(kern, (ncol + COLS - 1) / COLS, Cfg::THREADS, Cfg::SMEM, st, kDependent<R>, P.d, P.Sy[adj ? 1 : 0], w, P.tw[P.d.D - 1]);
 }
 template <typename R, int N> cudaError_t last2_n(const Plan<R>& P, cplx<R>* w, int adj, cudaStream_t st)
 {
     constexpr int CB = cols_big<R>(N), CS = cols_small<R>(N);
     const long long ncol = P.d.D == 3 ? (long long)P.d.n0 * P.d.n1 : P.d.n0;
-    if constexpr (CS < CB) {
-        if (small_tiles(ncol, CB)) return last2_tile<R, N, r_tile<R>(N), CS>(P, w, adj, st);
+    if constexpr (CS != CB || r_tile<R>(N) != r_axis<R>(N)) {
+        if (small_tiles<R, N>(ncol)) return last2_tile<R, N, r_tile<R>(N), CS>(P, w, adj, st);
     }
     return last2_tile<R, N, r_last<R>(N), CB>(P, w, adj, st);
 }
@@ -276,15 +322,15 @@ cudaError_t deriv_tile(const Plan<R>& P, const cplx<R>* x, cplx<R>* w, int e, in
     if (attr != cudaSuccess) return attr;
     const int n[3] = {P.d.n0, P.d.n1, P.d.n2};
     const long long ncol = P.d.N / n[e];
-    return launch(kern, (ncol + COLS - 1) / COLS, Cfg::THREADS, Cfg::SMEM, st, add != 0, P.d, P.L[adj ? 1 : 0], x, w, P.tw[e],
+    return launch(kern, (ncol + COLS - 1) / COLS, Cfg::THREADS, Cfg::SMEM, st, kDependent<R> && add != 0, P.d, P.L[adj ? 1 : 0], x, w, P.tw[e],
                   e, add);
 }
 template <typename R, int N>
 cudaError_t deriv_n(const Plan<R>& P, const cplx<R>* x, cplx<R>* w, int e, int add, int adj, cudaStream_t st)
 {
     constexpr int CB = cols_big<R>(N), CS = cols_small<R>(N);
-    if constexpr (CS < CB) {
-        if (small_tiles(P.d.N / N, CB)) return deriv_tile<R, N, r_tile<R>(N), CS>(P, x, w, e, add, adj, st);
+    if constexpr (CS != CB || r_tile<R>(N) != r_axis<R>(N)) {
+        if (small_tiles<R, N>(P.d.N / N)) return deriv_tile<R, N, r_tile<R>(N), CS>(P, x, w, e, add, adj, st);
     }
     return deriv_tile<R, N, r_axis<R>(N), CB>(P, x, w, e, add, adj, st);
 }
