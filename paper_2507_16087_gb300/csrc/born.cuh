@@ -280,8 +280,9 @@ template <typename R, int NX, int RX> struct RowCfg {
     static constexpr int UMAX = 64 / T < 2 ? 2 : 64 / T;
     static constexpr int UMIN = 32 / T < 2 ? 2 : 32 / T;  // whole warps
     static constexpr int MAXT = UMAX * T;
-    // float32: 128 registers a thread, 168 with 24 values
-    static constexpr int MINB = sizeof(R) == 4 ? (RX >= 24 ? 384 / MAXT : 512 / MAXT) : 1;
+    // float32: 128 registers a thread, 168 with 24 values, 72 with 8 (80 from 256 points: 72 spills there)
+    static constexpr int THREADS_SM = RX >= 24 ? 384 : (RX > 8 ? 512 : (NX >= 256 ? 768 : 896));
+    static constexpr int MINB = sizeof(R) == 4 ? THREADS_SM / MAXT : 1;
     // shared memory of a block of U units: x, w (and y), the medium rows (three a pair row), three barriers
     __host__ __device__ static constexpr size_t smem(int U, bool ysep)
     {

@@ -10,11 +10,11 @@
 namespace cbs {
 
 // Elements per thread of one transform.
-// float32 rows of 128 and more points: 16 values a thread (radix-16 passes: 128 = 16*8, 2048 = 16*16*8); float32
-// 3*2^k rows of 192 and more points: 24 (passes 3, 8, 8)
+// float32 rows: 8 values a thread up to 128 points (8*8*2 at 72 instead of 16*8 at 128 registers a thread: 55.4 instead of
+// 59.5 us at 128^3), 16 above (256^3 401 against 421 us, 512^3 3.55 against 4.16 ms). 3*2^k rows of 192 points: 24 (8*8*3).
 template <typename R> __host__ __device__ constexpr int r_rows(int n)
 {
-    return (n % 3 == 0) ? ((sizeof(R) == 4 && n >= 192) ? 24 : 12) : ((sizeof(R) == 4 && n >= 128) ? 16 : 8);
+    return (n % 3 == 0) ? ((sizeof(R) == 4 && n >= 192) ? 24 : 12) : ((sizeof(R) == 4 && n >= 256) ? 16 : 8);
 }
 // strided axes (two transforms a thread): 16 values for float32 axes of 128 and more points, else 8; 3*2^k: 12 (8 values
 // at 128^3 / 256^3 / 512^3: last axis 24.2 / 161 / 1581 us against 22.1 / 137 / 1471)
@@ -30,7 +30,11 @@ template <typename R> __host__ __device__ constexpr int r_tile(int n)
 {
     return sizeof(R) == 4 ? ((n % 3 == 0) ? 12 : 8) : ((n % 3 == 0) ? (n <= 48 ? 6 : 12) : (n <= 512 ? 4 : 8));
 }
-template <typename R> __host__ __device__ constexpr int r_rows_tile(int n) { return sizeof(R) == 4 ? r_rows<R>(n) : r_tile<R>(n); }
+// rows of small grids (see rows_tiny)
+template <typename R> __host__ __device__ constexpr int r_rows_tile(int n)
+{
+    return sizeof(R) == 4 ? (n == 512 ? 8 : r_rows<R>(n)) : r_tile<R>(n);
+}
 
 __host__ __device__ constexpr int max_i(int a, int b) { return a > b ? a : b; }
 // columns of a tile: whole 128-byte lines where a tile of two transforms leaves room for several blocks an SM (us of
@@ -114,10 +118,13 @@ template <typename R, int N, int RX> inline int rows_units_n(const Dims& d)
     while (u > Cfg::UMIN && units / u < kWaveBlocks) u /= 2;
     return u;
 }
-// values a thread of the row kernels on this grid: r_rows, or r_rows_tile when that leaves too few warps
+// whether the row kernels take r_rows_tile values a thread on this grid: float64 where r_rows leaves too few warps,
+// float32 512-point rows where all of them are on the SMs at once (512^2: 14.5 against 16.1 us an iteration)
 template <typename R, int N> inline bool rows_tiny(const Dims& d)
 {
-    return r_rows_tile<R>(N) < r_rows<R>(N) && few_warps<R>((long long)(d.D + 1) * d.N, r_rows<R>(N));
+    if (r_rows_tile<R>(N) >= r_rows<R>(N)) return false;
+    const long long values = (long long)(d.D + 1) * d.N;
+    return sizeof(R) == 8 ? few_warps<R>(values, r_rows<R>(N)) : values / r_rows<R>(N) <= 512LL * kSMs;
 }
 
 struct RowGrid {
