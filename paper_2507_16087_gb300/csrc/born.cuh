@@ -279,6 +279,10 @@ template <typename R, int NX, int RX> struct RowCfg {
     // 128^3, 421 against 410 us at 256^3)
     static constexpr int UMAX = 64 / T < 2 ? 2 : 64 / T;
     static constexpr int UMIN = 32 / T < 2 ? 2 : 32 / T;  // whole warps
+    // float32 rows of 1024 and more points: an SM holds too few of their large blocks to hide a second copy's wait
+    // behind each other, so y goes from global memory straight into registers (1024^2 36.7 -> 31.7, 2048^2 154 -> 129
+    // us; shorter rows lose: 128^3 55.3 against 58.3, 256^3 400 against 428)
+    static constexpr bool YREG = sizeof(R) == 4 && NX >= 1024;
     static constexpr int MAXT = UMAX * T;
     // float32: 128 registers a thread, 168 with 24 values, 72 with 8 (80 from 256 points: 72 spills there)
     static constexpr int THREADS_SM = RX >= 24 ? 384 : (RX > 8 ? 512 : (NX >= 256 ? 768 : 896));
@@ -326,13 +330,14 @@ k_rows(Dims d, Medium<R> M, Symbol<R> Sy, cplx<R>* __restrict__ x, const cplx<R>
     constexpr bool HAS_W = UPDATE || MODE == ROWS_GREEN;
     constexpr bool HAS_B = UPDATE || MODE == ROWS_FWD;  // B, y and the medium
     constexpr bool HAS_FWD = MODE == ROWS_FWD || MODE == ROWS_FUSED || MODE == ROWS_FUSED_NORM || MODE == ROWS_COPY;
+    constexpr bool YREG = UPDATE && RowCfg<R, NX, RX>::YREG;
     constexpr bool NORM = MODE == ROWS_FUSED_NORM || MODE == ROWS_INV;
     extern __shared__ __align__(128) unsigned char smraw[];
     const int U = blockDim.x / T, H = U >> 1;
     const int E = U * SL;
     CT* xs = reinterpret_cast<CT*>(smraw);
     CT* ws = xs + E;
-    const bool yown = UPDATE && ysep != 0;
+    const bool yown = UPDATE && !YREG && ysep != 0;
     CT* ys = yown ? ws + E : ws;
     R* ms = reinterpret_cast<R*>(ws + (yown ? 2 * E : E));
     uint64_t* bar = reinterpret_cast<uint64_t*>(ms + 3 * H * ML);
@@ -355,7 +360,7 @@ k_rows(Dims d, Medium<R> M, Symbol<R> Sy, cplx<R>* __restrict__ x, const cplx<R>
     if (isx) c = 0;
     const bool valid = lrow < nrow;
     const bool pres = pair && !isx;
-    constexpr int nbar = UPDATE ? 3 : 1;
+    constexpr int nbar = UPDATE ? (YREG ? 2 : 3) : 1;
     const long long v0 = row0 * NX;  // first voxel of the block's rows
     const int cs = pair ? d.D : c;   // component (slot) of the block's first array
     constexpr uint32_t FB = NX * sizeof(CT), MB = NX * sizeof(R);
@@ -382,7 +387,7 @@ k_rows(Dims d, Medium<R> M, Symbol<R> Sy, cplx<R>* __restrict__ x, const cplx<R>
             if constexpr (UPDATE) {
                 mbar_expect_tx(bar, fb);
                 mbar_expect_tx(bar + 1, two * fb + (pair ? 3u : 1u) * mb);
-                mbar_expect_tx(bar + 2, two * fb);
+                if constexpr (!YREG) mbar_expect_tx(bar + 2, two * fb);
             } else {
                 mbar_expect_tx(bar, 2u * two * fb + (pair ? 3u : 1u) * mb);
             }
@@ -458,11 +463,11 @@ k_rows(Dims d, Medium<R> M, Symbol<R> Sy, cplx<R>* __restrict__ x, const cplx<R>
         if constexpr (UPDATE) {
             // (the wait's barrier also ends every read of the exchange by the inverse transform)
             if (lost(1)) return;
-            if (!yown) {
+            if (!YREG && !yown) {
                 fence_proxy_async_smem();  // the generic-proxy accesses of the buffer come before the copies' writes
                 y_in(bar + 2);
             }
-            if (lost(2)) return;
+            if (!YREG && lost(2)) return;
         }
     } else if constexpr (HAS_B) {
         if (lost(0)) return;
@@ -472,12 +477,13 @@ k_rows(Dims d, Medium<R> M, Symbol<R> Sy, cplx<R>* __restrict__ x, const cplx<R>
         // the velocity's Pu (B x + y) in real space; the pressure has no such term
         const CT pu = pres ? mk<CT, R>((R)0, (R)0) : Sy.Pu;
         CT* xo = x + fbase + t;
+        const CT* yg = YREG ? y + fbase + t : yr;
         auto update = [&](auto is_pair) {
 #pragma unroll
             for (int s = 0; s < RX; ++s) {
                 const int o = T * slot_q<NX, RX, np>(s);
                 const CT bv = B_at(o, is_pair);
-                const CT xv = xr[o], yv = yr[o];
+                const CT xv = xr[o], yv = yg[o];
                 const CT wo = cfma(bv, xv, yv);                 // B x + y
                 const CT zx = cfma(pu, wo, csub(v[s], xv));     // z - x
                 const CT bn = cscale(bv, nu);
