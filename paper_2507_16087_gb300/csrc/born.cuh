@@ -75,11 +75,10 @@ template <typename R> struct Symbol {
     const R* k2[3];        // k_eta^2
 };
 
-// constants of L (off-diagonal i t_eta / sqrt(lambda1 lambda2)), forward or adjoint
+// off-diagonal factors of L per axis, i t_eta / (sqrt(lambda1 lambda2) n_eta) (the 1-D transforms' normalisation
+// included), negated for the adjoint
 template <typename R> struct LOp {
-    cplx<R> la1, la2;      // a_j / lambda_j
-    R g[3];                // +-1 / (sqrt(lambda1 lambda2) n_eta): sign - for the adjoint, 1-D normalisation included
-    const cplx<R>* kt[3];  // t_eta
+    const cplx<R>* it[3];
 };
 
 // Per-row view of B = 1 - v for component c (conj for the adjoint).  Along a
@@ -551,7 +550,9 @@ k_rows(Dims d, Medium<R> M, Symbol<R> Sy, cplx<R>* __restrict__ x, const cplx<R>
 template <typename R, int N, int RA, int COLS> struct PairCfg {
     static constexpr int T = N / RA;
     static constexpr int THREADS = T * COLS;
-    static constexpr size_t SMEM = plan_npass(N, RA) > 1 ? 2 * (size_t)N * COLS * sizeof(cplx<R>) : 0;
+    static constexpr bool PADC = COLS * sizeof(cplx<R>) < 128;
+    static constexpr int FSTRIDE = (PADC ? RowPad<cplx<R>, N, T>::pad(N - 1) + 1 : N) * COLS;  // values of one field's exchange
+    static constexpr size_t SMEM = plan_npass(N, RA) > 1 ? 2 * (size_t)FSTRIDE * sizeof(cplx<R>) : 0;
     // float32: 128 registers a thread
     static constexpr int MINB = sizeof(R) == 4 ? (THREADS >= 512 ? 1 : 512 / THREADS) : 1;
     static_assert(THREADS % 32 == 0 && THREADS <= 1024, "pair tile shape");
@@ -588,6 +589,7 @@ __global__ void __launch_bounds__(PairCfg<R, NA, RA, COLS>::THREADS, PairCfg<R, 
 k_axis2(Dims d, cplx<R>* __restrict__ w, const cplx<R>* __restrict__ tw, const cplx<R>* __restrict__ tab, int npair)
 {
     using CT = cplx<R>;
+    using Cfg = PairCfg<R, NA, RA, COLS>;
     constexpr int T = NA / RA;
     constexpr int np = plan_npass(NA, RA);
     extern __shared__ __align__(16) unsigned char smraw[];
@@ -615,7 +617,7 @@ k_axis2(Dims d, cplx<R>* __restrict__ w, const cplx<R>* __restrict__ tw, const c
 #pragma unroll
         for (int s = 0; s < RA; ++s) v[1][s] = cmul(v[0][s], __ldg(tab + t + T * slot_q<NA, RA, 0>(s)));
     }
-    fft_run_multi<NA, RA, 2, S, 0, true>(v, sm + col, COLS, NA * COLS, t, tw, BlockSync());
+    fft_run_multi<NA, RA, 2, S, Cfg::PADC>(v, sm + col, COLS, Cfg::FSTRIDE, t, tw, BlockSync());
     if (S < 0 && pair) {
 #pragma unroll
         for (int s = 0; s < RA; ++s) v[0][s] = cfma(v[1][s], __ldg(tab + t + T * slot_q<NA, RA, np>(s)), v[0][s]);
@@ -634,6 +636,7 @@ __global__ void __launch_bounds__(PairCfg<R, NL, RL, COLS>::THREADS, PairCfg<R, 
 k_last2(Dims d, Symbol<R> Sy, cplx<R>* __restrict__ w, const cplx<R>* __restrict__ tw)
 {
     using CT = cplx<R>;
+    using Cfg = PairCfg<R, NL, RL, COLS>;
     constexpr int T = NL / RL;
     constexpr int np = plan_npass(NL, RL);
     extern __shared__ __align__(16) unsigned char smraw[];
@@ -657,7 +660,7 @@ k_last2(Dims d, Symbol<R> Sy, cplx<R>* __restrict__ w, const cplx<R>* __restrict
     const CT* tm = d.D == 3 ? Sy.tm[2] : Sy.tm[1];
     const CT* td = d.D == 3 ? Sy.td[2] : Sy.td[1];
     const R* k2l = d.D == 3 ? Sy.k2[2] : Sy.k2[1];
-    fft_run_multi<NL, RL, 2, -1, 0, true>(v, sm + col, COLS, NL * COLS, t, tw, BlockSync());
+    fft_run_multi<NL, RL, 2, -1, Cfg::PADC>(v, sm + col, COLS, Cfg::FSTRIDE, t, tw, BlockSync());
 #pragma unroll
     for (int s = 0; s < RL; ++s) {
         const int k = t + T * slot_q<NL, RL, np>(s);
@@ -672,7 +675,7 @@ k_last2(Dims d, Symbol<R> Sy, cplx<R>* __restrict__ w, const cplx<R>* __restrict
     // the thread owns the same positions after the forward transform; reorder its registers into the entry order
     permute_slots<NL, RL, np, 0>(v[0]);
     permute_slots<NL, RL, np, 0>(v[1]);
-    fft_run_multi<NL, RL, 2, +1, 0, true>(v, sm + col, COLS, NL * COLS, t, tw, BlockSync());
+    fft_run_multi<NL, RL, 2, +1, Cfg::PADC>(v, sm + col, COLS, Cfg::FSTRIDE, t, tw, BlockSync());
     grid_trigger();
     if (valid) {
         col_store<NL, RL, np>(a, st, v[0]);
@@ -689,6 +692,7 @@ k_deriv2(Dims d, LOp<R> L, const cplx<R>* __restrict__ x, cplx<R>* __restrict__ 
          int e, int add)
 {
     using CT = cplx<R>;
+    using Cfg = PairCfg<R, N, RA, COLS>;
     constexpr int T = N / RA;
     constexpr int np = plan_npass(N, RA);
     extern __shared__ __align__(16) unsigned char smraw[];
@@ -708,18 +712,17 @@ k_deriv2(Dims d, LOp<R> L, const cplx<R>* __restrict__ x, cplx<R>* __restrict__ 
     grid_trigger_small<R>();
     col_load<N, RA, 0>(v[0], x + oa, st);
     col_load<N, RA, 0>(v[1], x + ob, st);
-    fft_run_multi<N, RA, 2, -1, 0, true>(v, sm + col, COLS, N * COLS, t, tw, BlockSync());
-    const CT* kt = e == 1 ? L.kt[1] : L.kt[2];
-    const R g = e == 1 ? L.g[1] : L.g[2];
+    fft_run_multi<N, RA, 2, -1, Cfg::PADC>(v, sm + col, COLS, Cfg::FSTRIDE, t, tw, BlockSync());
+    const CT* it = e == 1 ? L.it[1] : L.it[2];
 #pragma unroll
     for (int s = 0; s < RA; ++s) {
-        const CT f = mul_si<1>(cscale(__ldg(kt + t + T * slot_q<N, RA, np>(s)), g));  // i g t
+        const CT f = __ldg(it + t + T * slot_q<N, RA, np>(s));  // i g t
         v[0][s] = cmul(v[0][s], f);
         v[1][s] = cmul(v[1][s], mk<CT, R>(-f.x, f.y));  // i g conj(t) = -conj(i g t)
     }
     permute_slots<N, RA, np, 0>(v[0]);
     permute_slots<N, RA, np, 0>(v[1]);
-    fft_run_multi<N, RA, 2, +1, 0, true>(v, sm + col, COLS, N * COLS, t, tw, BlockSync());
+    fft_run_multi<N, RA, 2, +1, Cfg::PADC>(v, sm + col, COLS, Cfg::FSTRIDE, t, tw, BlockSync());
     if (valid) {
         col_store<N, RA, np>(w + ob, st, v[0]);
         if (add) {
@@ -733,7 +736,7 @@ k_deriv2(Dims d, LOp<R> L, const cplx<R>* __restrict__ x, cplx<R>* __restrict__ 
 
 // x axis of the operator and its diagonal: blocks as in k_rows (pair blocks transform p and u_x, the others only
 // combine), w on entry the gradients / divergence of k_deriv2.
-// OP_RESID: w <- y - A_s x, partial (|w|^2, |y|^2);  OP_APPLY: w <- A_s x, partial (|w|^2, 0).
+// OP_RESID: w <- y - A_s x, partial (|w|^2, |y|^2);  OP_APPLY: w <- A_s x, no partials.
 template <typename R, int NX, int RX>
 __global__ void __launch_bounds__(RowCfg<R, NX, RX>::MAXT, RowCfg<R, NX, RX>::MAXT <= 128 ? 3 : 1)
 k_rows_op(Dims d, Medium<R> M, LOp<R> L, const cplx<R>* __restrict__ x, const cplx<R>* __restrict__ y,
@@ -771,7 +774,6 @@ k_rows_op(Dims d, Medium<R> M, LOp<R> L, const cplx<R>* __restrict__ x, const cp
     const long long vbase = rest * NX;
     const long long fbase = (long long)c * d.N + vbase;
     const RowB<R> rb = row_B(M, d.D, c, i1, i2, vbase);
-    const CT la = pres ? L.la2 : L.la1;
     CT v[RX];
     grid_wait();
     grid_trigger_small<R>();
@@ -784,7 +786,7 @@ k_rows_op(Dims d, Medium<R> M, LOp<R> L, const cplx<R>* __restrict__ x, const cp
         fft_run<NX, RX, -1, true>(v, row, 1, t, tw, tc, RowSync<T>());
 #pragma unroll
         for (int s = 0; s < RX; ++s) {
-            CT f = mul_si<1>(cscale(__ldg(L.kt[0] + t + T * slot_q<NX, RX, np>(s)), L.g[0]));  // i g t
+            CT f = __ldg(L.it[0] + t + T * slot_q<NX, RX, np>(s));  // i g t
             if (isx) f.x = -f.x;
             v[s] = cmul(v[s], f);
         }
@@ -805,20 +807,30 @@ k_rows_op(Dims d, Medium<R> M, LOp<R> L, const cplx<R>* __restrict__ x, const cp
         for (int s = 0; s < RX; ++s) {
             const int i0 = t + T * slot_q<NX, RX, np>(s);
             const CT xv = x[fbase + i0];
-            const CT bv = born_B(M, rb, i0, adj != 0);
-            CT a = cfma(la, xv, csub(xv, cmul(bv, xv)));  // (a / lambda + v) x,  v = 1 - B
+            // the whole diagonal, a / lambda + v: rs (gamma + i omega), or kp ((gamma + et omega) + i (omega - gamma et))
+            const R g = __ldg(rb.g0 + i0) + rb.grest, m0 = __ldg(rb.m0 + i0);
+            CT dg;
+            if (pres) {
+                const R et = __ldg(rb.m1 + i0);
+                dg = mk<CT, R>(m0 * fma(et, M.omega, g), m0 * fma(-g, et, M.omega));
+            } else {
+                dg = mk<CT, R>(m0 * g, m0 * M.omega);
+            }
+            if (adj) dg.y = -dg.y;
+            CT a = mk<CT, R>((R)0, (R)0);
+            if (!isx) a = w[fbase + i0];
             if (pair) a = cadd(a, v[s]);
-            if (!isx) a = cadd(a, w[fbase + i0]);
+            a = cfma(dg, xv, a);
             if (mode == OP_RESID) {
                 const CT yv = y[fbase + i0];
                 a = csub(yv, a);
+                s0 += cabs2(a);
                 s1 += cabs2(yv);
             }
             w[fbase + i0] = a;
-            s0 += cabs2(a);
         }
     }
-    block_sum2(s0, s1, partials + 2 * (long long)blockIdx.x);
+    if (mode == OP_RESID) block_sum2(s0, s1, partials + 2 * (long long)blockIdx.x);
 }
 
 }  // namespace cbs

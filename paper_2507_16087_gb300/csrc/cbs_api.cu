@@ -528,14 +528,13 @@ struct cbs_solver {
     float *rs32[3] = {}, *kp32 = nullptr, *et32 = nullptr;
     double *gc64[3] = {}, *gs64[3] = {};
     float *gc32[3] = {}, *gs32[3] = {};
-    double2* kt64[3] = {};
     double* k264[3] = {};
     float2* kt32[3] = {};
     float* k232[3] = {};
     std::vector<double2> kt_host[3];
-    // merge / split factors of (L+I)^-1 per axis, [adjoint][axis]
-    double2 *tm64[2][3] = {}, *td64[2][3] = {};
-    float2 *tm32[2][3] = {}, *td32[2][3] = {};
+    // merge / split factors of (L+I)^-1 and off-diagonal factors of L per axis, [adjoint][axis]
+    double2 *tm64[2][3] = {}, *td64[2][3] = {}, *it64[2][3] = {};
+    float2 *tm32[2][3] = {}, *td32[2][3] = {}, *it32[2][3] = {};
     double2* tw64[3] = {};
     float2* tw32[3] = {};
 
@@ -1216,8 +1215,8 @@ void set_l2_window(cbs_solver* s, void* base, size_t bytes)
 
 using cd = std::complex<double>;
 
-// per-axis tables of (L+I)^-1 (top of born.cuh): tm = -(c1 / c2) conj(t), td = -Pu c1 / (l1 l2) t, forward and with
-// the constants conjugated for the adjoint
+// per-axis tables of (L+I)^-1 (top of born.cuh): tm = -(c1 / c2) conj(t), td = -Pu c1 / (l1 l2) t, and of L:
+// it = i t / (sqrt(l1 l2) n), forward and with the constants conjugated for the adjoint
 void green_tables(cbs_solver* s, TablePack& pack)
 {
     const double l1 = s->lam1, l2 = s->lam2;
@@ -1228,11 +1227,14 @@ void green_tables(cbs_solver* s, TablePack& pack)
         const cd fm = -(c1 / c2), fd = -pu * c1 / (l1 * l2);
         for (int a = 0; a < s->D; ++a) {
             const int n = s->n[a];
-            std::vector<double2> m(n), d(n);
-            std::vector<float2> m32(n), d32(n);
+            std::vector<double2> m(n), d(n), o(n);
+            std::vector<float2> m32(n), d32(n), o32(n);
+            const cd fo(0.0, (adj ? -1.0 : 1.0) / (std::sqrt(l1 * l2) * n));
             for (int i = 0; i < n; ++i) {
                 const cd t(s->kt_host[a][i].x, s->kt_host[a][i].y);
-                const cd tm = fm * std::conj(t), td = fd * t;
+                const cd tm = fm * std::conj(t), td = fd * t, it = fo * t;
+                o[i] = make_double2(it.real(), it.imag());
+                o32[i] = make_float2((float)it.real(), (float)it.imag());
                 m[i] = make_double2(tm.real(), tm.imag());
                 d[i] = make_double2(td.real(), td.imag());
                 m32[i] = make_float2((float)tm.real(), (float)tm.imag());
@@ -1242,6 +1244,8 @@ void green_tables(cbs_solver* s, TablePack& pack)
             pack.add(&s->td64[adj][a], d);
             pack.add(&s->tm32[adj][a], m32);
             pack.add(&s->td32[adj][a], d32);
+            pack.add(&s->it64[adj][a], o);
+            pack.add(&s->it32[adj][a], o32);
         }
     }
     pack.upload(s);
@@ -1269,7 +1273,7 @@ template <typename R> void fill_plan(cbs_solver* s, Plan<R>& P)
     P.M.a2r = (R)(s->a2r / s->lam2);
     P.M.a2i = (R)(s->a2i / s->lam2);
     // (L+I)^-1 (App. B.1 with a = a1, lambda_0 = lambda1, b = a2, lambda_1 = lambda2) and L
-    const double l1 = s->lam1, l2 = s->lam2, isq = 1.0 / std::sqrt(l1 * l2);
+    const double l1 = s->lam1, l2 = s->lam2;
     const cd a1l(s->a1r + l1, s->a1i), a2l(s->a2r + l2, s->a2i);
     auto c = [](cd v) { return mk<cplx<R>, R>((R)v.real(), (R)v.imag()); };
     for (int adj = 0; adj < 2; ++adj) {
@@ -1279,14 +1283,11 @@ template <typename R> void fill_plan(cbs_solver* s, Plan<R>& P)
         Y.c3 = cj(a1l * a2l);
         Y.cs = cj(l2 * a1l / (double)s->N);
         LOp<R>& L = P.L[adj];
-        L.la1 = cj(cd(s->a1r / l1, s->a1i / l1));
-        L.la2 = cj(cd(s->a2r / l2, s->a2i / l2));
         for (int e = 0; e < 3; ++e) {
             Y.tm[e] = f ? (const cplx<R>*)s->tm32[adj][e] : (const cplx<R>*)s->tm64[adj][e];
             Y.td[e] = f ? (const cplx<R>*)s->td32[adj][e] : (const cplx<R>*)s->td64[adj][e];
             Y.k2[e] = f ? (const R*)s->k232[e] : (const R*)s->k264[e];
-            L.kt[e] = f ? (const cplx<R>*)s->kt32[e] : (const cplx<R>*)s->kt64[e];
-            L.g[e] = (R)((adj ? -isq : isq) / s->n[e]);
+            L.it[e] = f ? (const cplx<R>*)s->it32[adj][e] : (const cplx<R>*)s->it64[adj][e];
         }
     }
 }
@@ -1465,7 +1466,6 @@ cbs_status solver_create(const cbs_grid* grid, double dx, double omega, const do
             pack.add(&s->gc64[a], gc);
             pack.add(&s->gs64[a], gs);
             pack.add(&s->k264[a], k2);
-            pack.add(&s->kt64[a], kt);
             pack.add(&s->tw64[a], tw);
             pack.add(&s->gc32[a], gc32);
             pack.add(&s->gs32[a], gs32);

@@ -425,24 +425,18 @@ __device__ __forceinline__ void pass_compute_multi(CT (&v)[C][R], int tid, const
     }
 }
 
-// Same for C independent transforms that share the thread mapping (used to
-// keep all components of a pencil in registers at once).
-// (twiddles read from the table: with C transforms in registers there is no
-// room to cache them; SHTW reads each one once for all C transforms)
-template <int N, int R, int C, int S, int P = 0, bool SHTW = false, typename CT, typename Sync>
+// C independent column transforms that share the thread mapping: each twiddle is read from the table once for all of
+// them (there is no room to keep twiddles in registers).  PADC: rows of the exchange at e + e / 16 (RowPad), for tiles
+// whose rows are shorter than 128 bytes: there the first pass's writes, 16 rows apart, would meet on the same banks.
+template <int N, int R, int C, int S, bool PADC, int P = 0, typename CT, typename Sync>
 __device__ __forceinline__ void fft_run_multi(CT (&v)[C][R], CT* sm, int ss, int cstride, int tid,
                                               const CT* __restrict__ tw, Sync sync)
 {
+    using L = RowPad<CT, N, N / R>;
     constexpr int T = N / R;
     constexpr int np = plan_npass(N, R);
     static_assert(np > 0, "unsupported FFT size / register split");
-    const TwCache<N, R, CT> none{};
-    if constexpr (SHTW) {
-        pass_compute_multi<N, R, T, P, S, C>(v, tid, tw);
-    } else {
-#pragma unroll
-        for (int c = 0; c < C; ++c) pass_compute<N, R, T, P, S, false>(v[c], tid, tw, none);
-    }
+    pass_compute_multi<N, R, T, P, S, C>(v, tid, tw);
     if constexpr (P + 1 < np) {
         constexpr int r = plan_radix(N, R, P);
         constexpr int NS = plan_ns(N, R, P);
@@ -455,7 +449,8 @@ __device__ __forceinline__ void fft_run_multi(CT (&v)[C][R], CT* sm, int ss, int
                 const int j = tid + T * m;
                 const int idx = (j / NS) * NS * r + (j % NS);
 #pragma unroll
-                for (int k = 0; k < r; ++k) sm[c * cstride + (idx + k * NS) * ss] = v[c][m * r + k];
+                for (int k = 0; k < r; ++k)
+                    sm[c * cstride + (PADC ? L::at(idx, k * NS) : idx + k * NS) * ss] = v[c][m * r + k];
             }
         sync();
 #pragma unroll
@@ -464,9 +459,10 @@ __device__ __forceinline__ void fft_run_multi(CT (&v)[C][R], CT* sm, int ss, int
             for (int m = 0; m < R / rn; ++m) {
                 const int j = tid + T * m;
 #pragma unroll
-                for (int k = 0; k < rn; ++k) v[c][m * rn + k] = sm[c * cstride + (j + k * (N / rn)) * ss];
+                for (int k = 0; k < rn; ++k)
+                    v[c][m * rn + k] = sm[c * cstride + (PADC ? L::at(j, k * (N / rn)) : j + k * (N / rn)) * ss];
             }
-        fft_run_multi<N, R, C, S, P + 1, SHTW>(v, sm, ss, cstride, tid, tw, sync);
+        fft_run_multi<N, R, C, S, PADC, P + 1>(v, sm, ss, cstride, tid, tw, sync);
     }
 }
 
