@@ -283,8 +283,9 @@ template <typename R, int NX, int RX> struct RowCfg {
     // us; shorter rows lose: 128^3 55.3 against 58.3, 256^3 400 against 428)
     static constexpr bool YREG = sizeof(R) == 4 && NX >= 1024;
     static constexpr int MAXT = UMAX * T;
-    // float32: 128 registers a thread, 168 with 24 values, 72 with 8 (80 from 256 points: 72 spills there)
-    static constexpr int THREADS_SM = RX >= 24 ? 384 : (RX > 8 ? 512 : (NX >= 256 ? 768 : 896));
+    // float32: 128 registers a thread with 16 values, 88 with 12 (96^3 30.8 against 34.7 us at 128, 192^3 209 against 221),
+    // 72 with 8 (80 from 256 points: 72 spills there)
+    static constexpr int THREADS_SM = RX > 12 ? 512 : (RX > 8 ? 704 : (NX >= 256 ? 768 : 896));
     static constexpr int MINB = sizeof(R) == 4 ? THREADS_SM / MAXT : 1;
     // shared memory of a block of U units: x, w (and y), the medium rows (three a pair row), three barriers
     __host__ __device__ static constexpr size_t smem(int U, bool ysep)

@@ -171,15 +171,16 @@ __global__ void k_setup_minmax(SetupIn s, double* part, int* bad)
         for (int k = 0; k < 8; ++k) part[blockIdx.x * 8 + k] = sh[k][0];
 }
 
-// per block: max |d - a1|, max |q - a2|
-__global__ void k_setup_maxdev(SetupIn s, double2 a1, double2 a2, double* part)
+// per block: max |(d - a1) s1|^2, max |(q - a2) s2|^2 (squares: a hypot is tens of FP64 instructions; the scales s_j, about
+// 1 / |a_j|, keep them from over- and underflow whatever the medium's units)
+__global__ void k_setup_maxdev(SetupIn s, double2 a1, double2 a2, double s1, double s2, double* part)
 {
     double m1 = 0.0, m2 = 0.0;
     for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < s.N; i += (long long)gridDim.x * blockDim.x) {
         double2 d[3], q;
         diag_values(s, i, d, q);
-        for (int e = 0; e < s.D; ++e) m1 = fmax(m1, hypot(d[e].x - a1.x, d[e].y - a1.y));
-        m2 = fmax(m2, hypot(q.x - a2.x, q.y - a2.y));
+        for (int e = 0; e < s.D; ++e) m1 = fmax(m1, cabs2(cscale(csub(d[e], a1), s1)));
+        m2 = fmax(m2, cabs2(cscale(csub(q, a2), s2)));
     }
     __shared__ double sh[2][kSetupThreads];
     sh[0][threadIdx.x] = m1;
@@ -1540,12 +1541,20 @@ cbs_status solver_create(const cbs_grid* grid, double dx, double omega, const do
             dfree(s, qv);
         }
         TRACE("create: maxdev");
-        k_setup_maxdev<<<sg, kSetupThreads, 0, s->st>>>(si, make_double2(s->a1r, s->a1i), make_double2(s->a2r, s->a2i), part);
+        auto scale_of = [](double re, double im) {
+            const double m = std::hypot(re, im);
+            return m > 0 && std::isfinite(1.0 / m) ? m : 1.0;
+        };
+        const double f1 = scale_of(s->a1r, s->a1i), f2 = scale_of(s->a2r, s->a2i);
+        k_setup_maxdev<<<sg, kSetupThreads, 0, s->st>>>(si, make_double2(s->a1r, s->a1i), make_double2(s->a2r, s->a2i), 1.0 / f1,
+                                                        1.0 / f2, part);
         CUDA_TRY(cudaGetLastError());
         CUDA_TRY(cudaMemcpyAsync(hp.data(), part, (size_t)sg * 2 * sizeof(double), cudaMemcpyDeviceToHost, s->st));
         CUDA_TRY(cudaStreamSynchronize(s->st));
         double m1 = 0, m2 = 0;
         for (int bi = 0; bi < sg; ++bi) { m1 = std::max(m1, hp[bi * 2]); m2 = std::max(m2, hp[bi * 2 + 1]); }
+        m1 = std::sqrt(m1) * f1;
+        m2 = std::sqrt(m2) * f2;
         s->lam1 = m1 > 0 ? m1 / o.beta : std::hypot(s->a1r, s->a1i);
         s->lam2 = m2 > 0 ? m2 / o.beta : std::hypot(s->a2r, s->a2i);
         if (!(s->lam1 > 0) || !(s->lam2 > 0) || !std::isfinite(s->lam1) || !std::isfinite(s->lam2)) {

@@ -11,10 +11,10 @@ namespace cbs {
 
 // Elements per thread of one transform.
 // float32 rows: 8 values a thread up to 128 points (8*8*2 at 72 instead of 16*8 at 128 registers a thread: 55.4 instead of
-// 59.5 us at 128^3), 16 above (256^3 401 against 421 us, 512^3 3.55 against 4.16 ms). 3*2^k rows of 192 points: 24 (8*8*3).
+// 59.5 us at 128^3), 16 above (256^3 401 against 421 us, 512^3 3.55 against 4.16 ms). 3*2^k rows: 12 (192^3 209 against 221 us with 24).
 template <typename R> __host__ __device__ constexpr int r_rows(int n)
 {
-    return (n % 3 == 0) ? ((sizeof(R) == 4 && n >= 192) ? 24 : 12) : ((sizeof(R) == 4 && n >= 256) ? 16 : 8);
+    return (n % 3 == 0) ? 12 : ((sizeof(R) == 4 && n >= 256) ? 16 : 8);
 }
 // strided axes (two transforms a thread): 16 values for float32 axes of 128 and more points, else 8; 3*2^k: 12 (8 values
 // at 128^3 / 256^3 / 512^3: last axis 24.2 / 161 / 1581 us against 22.1 / 137 / 1471)
