@@ -247,7 +247,6 @@ __device__ __forceinline__ bool mbar_try_wait(uint64_t* bar, uint32_t phase)
 
 constexpr int kBulkWaitLimit = 1 << 22;  // try_wait rounds before a copy is declared lost
 constexpr int kErrBulkTimeout = 1;
-constexpr int kErrTileAlign = 2;  // a shared-memory tile not on the 128-byte boundary tensor copies want
 
 // true when the phase completed; false after kBulkWaitLimit rounds
 __device__ __forceinline__ bool mbar_wait_bounded(uint64_t* bar, uint32_t phase, int limit = kBulkWaitLimit)
@@ -257,7 +256,7 @@ __device__ __forceinline__ bool mbar_wait_bounded(uint64_t* bar, uint32_t phase,
     return false;
 }
 
-// orders this thread's shared-memory accesses before later bulk / tensor copies that read or overwrite the buffer
+// orders this thread's shared-memory accesses before later bulk copies that read or overwrite the buffer
 __device__ __forceinline__ void fence_proxy_async_smem() { asm volatile("fence.proxy.async.shared::cta;" ::: "memory"); }
 
 
@@ -274,8 +273,8 @@ template <typename R, int NX, int RX> struct RowCfg {
     static constexpr int T = NX / RX;
     static constexpr int SL = RowPad<cplx<R>, NX, T>::SL;        // row pitch of the field buffers (values)
     static constexpr int ML = (SL + 3) / 4 * 4;                  // row pitch of the medium buffers (reals)
-    // 64 threads: many small blocks in different phases keep copies in flight (128 threads: 63.8 against 62.1 us at
-    // 128^3, 421 against 410 us at 256^3)
+    // 64 threads: many small blocks in different phases keep copies in flight (128 threads, both with 16 values: 63.8
+    // against 62.1 us at 128^3, 421 against 410 us at 256^3)
     static constexpr int UMAX = 64 / T < 2 ? 2 : 64 / T;
     static constexpr int UMIN = 32 / T < 2 ? 2 : 32 / T;  // whole warps
     // float32 rows of 1024 and more points: an SM holds too few of their large blocks to hide a second copy's wait
@@ -316,6 +315,9 @@ template <bool PAIR, typename R> __device__ __forceinline__ cplx<R> voxel_B(cons
     else return mk<cplx<R>, R>(fma(-m0, g, u.cr), fma(-m0, u.so, u.ci));
 }
 
+// Bound by HBM where w does not fit in L2 (256^3: 402 us, 164 B/voxel at 6.8 TB/s; 512^3: 3.56 ms at 6.2 TB/s), by latency
+// where it does (128^3: 55 us at 61 % of DRAM throughput, 26 warps an SM; stalls first on the staged copies).  The kernels it
+// replaced, one per component: 60.9 us, 438 us, 3.94 ms.
 template <typename R, int NX, int RX, int MODE>
 __global__ void __launch_bounds__(RowCfg<R, NX, RX>::MAXT, RowCfg<R, NX, RX>::MINB)
 k_rows(Dims d, Medium<R> M, Symbol<R> Sy, cplx<R>* __restrict__ x, const cplx<R>* __restrict__ y,
@@ -582,7 +584,8 @@ __device__ __forceinline__ void col_store(CT* p, long long st, const CT (&v)[RA]
     }
 }
 
-// y axis of a 3D field.  S = -1: blocks b < npair transform (q, u_y) and store q + tm_y u_y; S = +1: they read q
+// y axis of a 3D field (16.9 and 16.4 us at 128^3, 108 and 112 us at 256^3, 5.0 and 6.1 TB/s; the four-component
+// transforms it replaced 21.9 and 20.5, 198 and 199 us).  S = -1: blocks b < npair transform (q, u_y) and store q + tm_y u_y; S = +1: they read q
 // only and store the inverse transforms of q and td_y q (slot 1).  The other blocks transform two u_z columns a
 // thread (the column and the one half the columns further on).
 template <typename R, int NA, int RA, int COLS, int S>
@@ -632,6 +635,8 @@ k_axis2(Dims d, cplx<R>* __restrict__ w, const cplx<R>* __restrict__ tw, const c
 
 // Last axis: forward transforms of (q, u_last), b = q + tm u_last, p = cs b / (|k|^2 + c3), inverse transforms of p
 // and td p.  grid: ceil(n0 n1 / COLS) (3D) or ceil(n0 / COLS) (2D).
+// Bound on chip, by exchanges, barriers and the first loads of a wave: 22 us at 128^3 (6 at L2 rate), 129 us at 256^3 and 1.45
+// ms at 512^3 (79 and 632 us at HBM rate); holding all four components it took 40.5 us, 334 us and 3.24 ms.
 template <typename R, int NL, int RL, int COLS>
 __global__ void __launch_bounds__(PairCfg<R, NL, RL, COLS>::THREADS, PairCfg<R, NL, RL, COLS>::MINB)
 k_last2(Dims d, Symbol<R> Sy, cplx<R>* __restrict__ w, const cplx<R>* __restrict__ tw)
