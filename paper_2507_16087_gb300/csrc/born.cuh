@@ -268,7 +268,7 @@ __device__ __forceinline__ void fence_proxy_async_smem() { asm volatile("fence.p
 // exchange runs in the staged w row and the rows that share a shared-memory phase lie on different banks.
 // y lands in w's rows once the inverse transform has been read out of them (ysep = 0: two field buffers a block,
 // more blocks an SM) or in a buffer of its own, issued at the start (ysep = 1: small grids, where a block's
-// chain of waits is the time).  The two modes without B (ROWS_COPY, ROWS_GREEN) load straight from global memory.
+// chain of waits is the time); rows of 1024 and more float32 points have no such buffer (YREG).  The two modes without B (ROWS_COPY, ROWS_GREEN) load straight from global memory.
 template <typename R, int NX, int RX> struct RowCfg {
     static constexpr int T = NX / RX;
     static constexpr int SL = RowPad<cplx<R>, NX, T>::SL;        // row pitch of the field buffers (values)
@@ -286,10 +286,18 @@ template <typename R, int NX, int RX> struct RowCfg {
     // 72 with 8 (80 from 256 points: 72 spills there)
     static constexpr int THREADS_SM = RX > 12 ? 512 : (RX > 8 ? 704 : (NX >= 256 ? 768 : 896));
     static constexpr int MINB = sizeof(R) == 4 ? THREADS_SM / MAXT : 1;
-    // shared memory of a block of U units: x, w (and y), the medium rows (three a pair row), three barriers
-    __host__ __device__ static constexpr size_t smem(int U, bool ysep)
+    // whether the mode's y may have a buffer of its own (ysep): the updates, unless y goes to registers
+    __host__ __device__ static constexpr bool own_y(int mode)
     {
-        return (size_t)U * SL * sizeof(cplx<R>) * (ysep ? 3 : 2) + (size_t)U / 2 * 3 * ML * sizeof(R) + 32;
+        return !YREG && (mode == ROWS_FUSED || mode == ROWS_FUSED_NORM || mode == ROWS_INV);
+    }
+    // shared memory of a block of U units: x, w (and y), the medium rows (three a pair row), three barriers; the two
+    // modes without B take the exchange only
+    __host__ __device__ static constexpr size_t smem(int U, int mode, bool ysep)
+    {
+        const size_t field = (size_t)U * SL * sizeof(cplx<R>);
+        if (mode == ROWS_COPY || mode == ROWS_GREEN) return field;
+        return field * (own_y(mode) && ysep ? 3 : 2) + (size_t)U / 2 * 3 * ML * sizeof(R) + 32;
     }
 };
 
@@ -338,8 +346,8 @@ k_rows(Dims d, Medium<R> M, Symbol<R> Sy, cplx<R>* __restrict__ x, const cplx<R>
     const int U = blockDim.x / T, H = U >> 1;
     const int E = U * SL;
     CT* xs = reinterpret_cast<CT*>(smraw);
-    CT* ws = xs + E;
-    const bool yown = UPDATE && !YREG && ysep != 0;
+    CT* ws = HAS_B ? xs + E : xs;
+    const bool yown = Cfg::own_y(MODE) && ysep != 0;
     CT* ys = yown ? ws + E : ws;
     R* ms = reinterpret_cast<R*>(ws + (yown ? 2 * E : E));
     uint64_t* bar = reinterpret_cast<uint64_t*>(ms + 3 * H * ML);

@@ -160,17 +160,20 @@ cudaError_t rows_nm(const Plan<R>& P, cplx<R>* x, const cplx<R>* y, cplx<R>* w, 
 {
     using Cfg = RowCfg<R, N, RX>;
     auto kern = k_rows<R, N, RX, MODE>;
+    constexpr bool kOwnY = Cfg::own_y(MODE) && Cfg::smem(Cfg::UMAX, MODE, true) < kMaxDynSmem;
     // once per process, thread-safe (function-local static)
-    static const cudaError_t attr = cudaFuncSetAttribute(
-        kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
-        (int)(Cfg::smem(Cfg::UMAX, true) < kMaxDynSmem ? Cfg::smem(Cfg::UMAX, true) : Cfg::smem(Cfg::UMAX, false)));
+    static const cudaError_t attr = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                                         (int)Cfg::smem(Cfg::UMAX, MODE, kOwnY));
     if (attr != cudaSuccess) return attr;
     const RowGrid g = row_grid<R, N>(P.d);
-    // a grid of few blocks an SM gives y a buffer of its own, its copy in flight from the start (64^3: 12.3 against
-    // 14.1 us; above that the room costs more blocks than the wait does time: 192^3 331 against 296 us)
-    const int ysep = g.blocks <= 4 * kWaveBlocks && Cfg::smem(g.units, true) < kMaxDynSmem ? 1 : 0;
+    // a grid of few blocks an SM gives y a buffer of its own, its copy in flight from the start (us an iteration: 128^2
+    // 7.4 against 8.1, 256^2 8.9 against 9.5, 512^2 with 768 blocks 14.0 against 14.5); above that the room costs more
+    // blocks than the wait does time (192^3 rows 331 against 296 us).  No block takes a buffer that its mode or row
+    // length does not use: with y's, 1024- and 2048-point rows ran three and one blocks an SM in place of four and two
+    // (96 x 2048 22.1 against 18.6 us an iteration, 512 x 2048 60.9 against 50.6)
+    const int ysep = kOwnY && g.blocks <= 4 * kWaveBlocks ? 1 : 0;
     // the modes that start a chain follow other work (x and y may have just been written)
-    return launch(kern, g.blocks, g.units * Cfg::T, Cfg::smem(g.units, ysep != 0), st,
+    return launch(kern, g.blocks, g.units * Cfg::T, Cfg::smem(g.units, MODE, ysep != 0), st,
                   kDependent<R> && MODE != ROWS_FWD && MODE != ROWS_COPY, P.d, P.M, P.Sy[adj ? 1 : 0], x, y, w, P.tw[0], g.npair, g.nsingle, ysep, adj, nu, partials, P.err);
 }
 

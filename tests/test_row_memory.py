@@ -1,0 +1,94 @@
+"""Shared memory the row kernels' launches ask for (csrc/launch.cuh), on the CPU: the launchers run against a stand-in
+for the runtime's launch call that records each launch.  A block must not take room that its mode or row length never
+touches, or fewer blocks fit on an SM than the kernel was compiled for."""
+import ctypes
+import os
+import shutil
+import subprocess
+import tempfile
+
+import pytest
+
+ROOT = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
+CSRC = os.path.join(ROOT, "paper_2507_16087_gb300", "csrc")
+FWD, FUSED, FUSED_NORM, INV, COPY, GREEN = range(6)  # RowsMode
+
+SRC = r'''
+#include <cuda_runtime.h>
+static int g_threads, g_smem, g_blocks;
+extern "C" cudaError_t cudaLaunchKernelExC(const cudaLaunchConfig_t* c, const void*, void**)
+{ g_threads = c->blockDim.x; g_smem = (int)c->dynamicSmemBytes; g_blocks = c->gridDim.x; return cudaSuccess; }
+extern "C" cudaError_t cudaFuncSetAttribute(const void*, cudaFuncAttribute, int) { return cudaSuccess; }
+#include "launch.cuh"
+using namespace cbs;
+
+template <typename R, int N> int run(int D, int n1, int n2, int mode, int* o)
+{
+    Plan<R> P{};
+    P.d.D = D; P.d.n0 = N; P.d.n1 = n1; P.d.n2 = n2; P.d.N = (long long)N * n1 * n2;
+    const bool tiny = rows_tiny<R, N>(P.d);
+    const cudaError_t e = rows_n<R, N>(P, nullptr, nullptr, nullptr, mode, 0, (R)0, nullptr, nullptr);
+    using A = RowCfg<R, N, r_rows<R>(N)>;
+    using B = RowCfg<R, N, r_rows_tile<R>(N)>;
+    o[0] = g_threads; o[1] = g_smem; o[2] = g_blocks;
+    o[3] = tiny ? B::MINB : A::MINB;                       // blocks an SM the kernel is compiled for
+    o[4] = (tiny ? B::SL : A::SL) * (int)sizeof(cplx<R>);  // a field row
+    o[5] = (tiny ? B::ML : A::ML) * (int)sizeof(R);        // a medium row
+    o[6] = g_threads / (tiny ? B::T : A::T);               // units
+    return (int)e;
+}
+extern "C" int row_launch(int f64, int D, int n0, int n1, int n2, int mode, int* o)
+{
+    if (!f64 && n0 == 2048) return run<float, 2048>(D, n1, n2, mode, o);
+    if (!f64 && n0 == 1024) return run<float, 1024>(D, n1, n2, mode, o);
+    if (!f64 && n0 == 64) return run<float, 64>(D, n1, n2, mode, o);
+    if (f64 && n0 == 64) return run<double, 64>(D, n1, n2, mode, o);
+    return -1;
+}
+'''
+
+
+@pytest.fixture(scope="module")
+def lib():
+    nvcc = shutil.which("nvcc") or "/usr/local/cuda/bin/nvcc"
+    d = tempfile.mkdtemp()
+    src, so = os.path.join(d, "mem.cu"), os.path.join(d, "mem.so")
+    open(src, "w").write(SRC)
+    # PTX only (nothing here runs on a device); the shared runtime and references bound within the library, so that the
+    # stand-ins above take the place of its calls
+    subprocess.check_call([nvcc, "-std=c++17", "-gencode", "arch=compute_103a,code=compute_103a", "-cudart", "shared",
+                           "-Xlinker", "-Bsymbolic", "-Xcompiler", "-fPIC", "-shared", "-I" + CSRC, "-I" + os.path.join(ROOT, "include"), src,
+                           "-o", so])
+    L = ctypes.CDLL(so)
+    L.row_launch.argtypes = [ctypes.c_int] * 6 + [ctypes.c_void_p]
+    return L
+
+
+def launched(lib, f64, grid, mode):
+    D = len(grid)
+    o = (ctypes.c_int * 7)()
+    assert lib.row_launch(f64, D, grid[0], grid[1], grid[2] if D == 3 else 1, mode, o) == 0
+    return dict(zip(("threads", "smem", "blocks", "minb", "row", "mrow", "units"), o))
+
+
+@pytest.mark.parametrize("grid", [(2048, 64), (2048, 512), (2048, 2048), (1024, 12), (1024, 512), (1024, 1024),
+                                  (1024, 8, 16), (2048, 8, 8)])
+@pytest.mark.parametrize("mode", [FWD, FUSED, FUSED_NORM, INV])
+def test_long_rows_fit_the_blocks_an_sm_they_are_compiled_for(lib, grid, mode):
+    g = launched(lib, 0, grid, mode)
+    assert g["minb"] >= 2
+    # 228 KiB of shared memory an SM; 1 KiB of it and the norms' 512 B of static scratch go with each block
+    assert g["minb"] * (g["smem"] + 1024 + 512) <= 228 * 1024
+
+
+@pytest.mark.parametrize("f64,grid", [(0, (2048, 64)), (0, (1024, 2048)), (0, (64, 12)), (0, (64, 64, 64)), (1, (64, 12)),
+                                      (1, (64, 64, 64))])
+@pytest.mark.parametrize("mode", range(6))
+def test_a_launch_asks_for_the_buffers_its_mode_uses(lib, f64, grid, mode):
+    g = launched(lib, f64, grid, mode)
+    fields = 1 if mode in (COPY, GREEN) else 2  # x and w; only the exchange in the modes without B
+    medium = 0 if mode in (COPY, GREEN) else g["units"] // 2 * 3 * g["mrow"]
+    least = g["units"] * fields * g["row"] + medium
+    # y may have a buffer of its own in the updates, for rows whose y is staged; the barriers take up to 32 bytes
+    own_y = g["units"] * g["row"] if mode in (FUSED, FUSED_NORM, INV) and not (grid[0] >= 1024 and not f64) else 0
+    assert g["smem"] in (least, least + 32, least + own_y + 32)
