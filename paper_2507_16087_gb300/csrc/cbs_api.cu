@@ -347,71 +347,82 @@ struct ScaleIn {
     const double* kp;
     const double* et;
     double sl1, sl2;  // sqrt(lambda1), sqrt(lambda2)
+    double il1, il2;  // their reciprocals
 };
 
 // y = C^-1/2 s_hat,  s_hat_u = (S+ rho) s_u,  s_hat_p = s_p / (rho c^2)
 // (rs sqrt(l1) = (S+ rho)/sqrt(l1);  kp sqrt(l2) (1 - i et) = 1/(rho c^2 sqrt(l2)))
-// value i of component c of the scaled source.  Sources are points and bowls in earnest: a zero costs no FP64 instruction
-// (an SM issues them at 1/64 of its float32 rate, so dense arithmetic here takes longer than the memory).
+// Sources are points and bowls in earnest, or dense (adjoint right-hand sides of whole fields, residuals): a zero reads no
+// medium and costs no FP64 instruction (an SM issues those at 1/64 of its float32 rate).
 __device__ __forceinline__ bool is_zero(double2 v)
 {
     return ((__double_as_longlong(v.x) | __double_as_longlong(v.y)) << 1) == 0;
 }
-__device__ __forceinline__ double2 scaled_source(const ScaleIn& p, double2 v, int c, long long i, int adjoint)
-{
-    if (adjoint) {
-        const double f = 1.0 / (c < p.D ? p.sl1 : p.sl2);
-        return make_double2(v.x * f, v.y * f);
-    }
-    if (c < p.D) {
-        const double f = p.rs[c][i] * p.sl1;
-        return make_double2(v.x * f, v.y * f);
-    }
-    const double k = p.kp[i] * p.sl2, e = p.et[i];
-    return make_double2(k * (v.x + e * v.y), k * (v.y - e * v.x));  // v * k (1 - i e)
-}
 
-// grids of these kernels: x over voxels, y the component
-__global__ void k_scale_source(ScaleIn p, const double2* __restrict__ src, double2* __restrict__ y, int adjoint)
+enum SourceKind { SRC_VELOCITY, SRC_PRESSURE, SRC_ADJOINT };
+// A value of one kind from the source's; m and et at its medium values.  Not inlined: an FP64 instruction takes its issue
+// slots whether or not its predicate holds, and only around a call does the compiler branch in place of predicating (us at
+// 256^3, 316 at HBM rate without the medium: dense forward 1029 with the kinds predicated in one loop, 479 so; sparse 442
+// with the zeros predicated, 327 so).
+template <int KIND> __device__ __noinline__ double2 scaled_value(double2 v, const double* m, const double* et, double sl)
+{
+    if constexpr (KIND == SRC_ADJOINT) return make_double2(v.x * sl, v.y * sl);
+    const double g = *m * sl;
+    if constexpr (KIND == SRC_VELOCITY) return make_double2(v.x * g, v.y * g);
+    const double e = *et;
+    return make_double2(g * (v.x + e * v.y), g * (v.y - e * v.x));  // v g (1 - i e)
+}
+// this block's values i of one component, two at a time (their loads go together): zero(i, v) where the source is zero,
+// else value(i, y_i)
+template <int KIND, typename Zero, typename Value>
+__device__ __forceinline__ void for_component(long long N, const double2* __restrict__ s, const double* __restrict__ m0,
+                                              const double* __restrict__ et, double sl, Zero zero, Value value)
+{
+    const long long st = (long long)gridDim.x * blockDim.x;
+    for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < N; i += 2 * st) {
+        const long long j = i + st;
+        const double2 v = s[i], u = j < N ? s[j] : make_double2(0.0, 0.0);
+        if (is_zero(v)) zero(i, v);
+        else value(i, scaled_value<KIND>(v, m0 + i, et + i, sl));
+        if (j < N) {
+            if (is_zero(u)) zero(j, u);
+            else value(j, scaled_value<KIND>(u, m0 + j, et + j, sl));
+        }
+    }
+}
+// the scaled source's component c = blockIdx.y (grids: x over voxels, y the component)
+template <typename Zero, typename Value>
+__device__ __forceinline__ void for_scaled_source(const ScaleIn& p, const double2* __restrict__ src, int adjoint, Zero zero,
+                                                  Value value)
 {
     const int c = blockIdx.y;
-    const long long o = (long long)c * p.N;
-    for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < p.N; i += (long long)gridDim.x * blockDim.x) {
-        double2 v = src[o + i];
-        if (!is_zero(v)) v = scaled_source(p, v, c, i, adjoint);
-        y[o + i] = v;
-    }
+    const double2* s = src + (long long)c * p.N;
+    if (adjoint) for_component<SRC_ADJOINT>(p.N, s, nullptr, nullptr, c < p.D ? p.il1 : p.il2, zero, value);
+    else if (c < p.D) for_component<SRC_VELOCITY>(p.N, s, c == 0 ? p.rs[0] : (c == 1 ? p.rs[1] : p.rs[2]), nullptr, p.sl1, zero, value);
+    else for_component<SRC_PRESSURE>(p.N, s, p.kp, p.et, p.sl2, zero, value);
+}
+
+__global__ void k_scale_source(ScaleIn p, const double2* __restrict__ src, double2* __restrict__ y, int adjoint)
+{
+    double2* yc = y + (long long)blockIdx.y * p.N;
+    auto store = [&](long long i, double2 v) { yc[i] = v; };
+    for_scaled_source(p, src, adjoint, store, store);
 }
 
 // the float32 path's right-hand side straight from the source: y32 = (float)(s y)
 __global__ void k_scale_source_32(ScaleIn p, const double2* __restrict__ src, float2* __restrict__ y, double s, int adjoint)
 {
-    const int c = blockIdx.y;
-    const long long o = (long long)c * p.N;
-    for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < p.N; i += (long long)gridDim.x * blockDim.x) {
-        double2 v = src[o + i];
-        float2 r = make_float2(0.0f, 0.0f);
-        if (!is_zero(v)) {
-            v = scaled_source(p, v, c, i, adjoint);
-            r = make_float2((float)(v.x * s), (float)(v.y * s));
-        }
-        y[o + i] = r;
-    }
+    float2* yc = y + (long long)blockIdx.y * p.N;
+    for_scaled_source(p, src, adjoint, [&](long long i, double2) { yc[i] = make_float2(0.0f, 0.0f); },
+                      [&](long long i, double2 v) { yc[i] = make_float2((float)(v.x * s), (float)(v.y * s)); });
 }
 
 // per-block partial sums of |y|^2 of the scaled source (grid-stride, fixed assignment -> deterministic)
 __global__ void k_source_norm2(ScaleIn p, const double2* __restrict__ src, int adjoint, double* part)
 {
-    const int c = blockIdx.y;
-    const long long o = (long long)c * p.N;
     double s = 0.0;
-    for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < p.N; i += (long long)gridDim.x * blockDim.x) {
-        double2 v = src[o + i];
-        if (!is_zero(v)) {
-            v = scaled_source(p, v, c, i, adjoint);
-            s += v.x * v.x + v.y * v.y;
-        }
-    }
+    for_scaled_source(p, src, adjoint, [](long long, double2) {},
+                      [&](long long, double2 v) { s += v.x * v.x + v.y * v.y; });
     block_sum2(s, 0.0, part + 2 * (blockIdx.y * gridDim.x + blockIdx.x));
 }
 
@@ -838,19 +849,23 @@ ScaleIn scale_in(cbs_solver* s)
     p.et = s->et64;
     p.sl1 = std::sqrt(s->lam1);
     p.sl2 = std::sqrt(s->lam2);
+    p.il1 = 1.0 / p.sl1;
+    p.il2 = 1.0 / p.sl2;
     return p;
 }
 
 long long field_len(cbs_solver* s) { return (long long)s->C * s->N; }
 
-// x over voxels (as many blocks as one component needs of grid_for's), y the component
+// grids of the kernels over voxels (x) and components (y): as many blocks as one component needs of grid_for's, and C
+// times as many for scaling the source on small grids (there every block's partial sum would cost the norm more)
 dim3 voxel_grid(cbs_solver* s) { return dim3((unsigned)std::max(1, grid_for(s->N) / s->C), (unsigned)s->C); }
+dim3 scale_grid(cbs_solver* s) { return dim3((unsigned)std::max(1, grid_for(s->C * s->N) / s->C), (unsigned)s->C); }
 
 // physical source -> y64 ; optional start field -> x64 (C^1/2 (u,p)) else 0
 void prepare(cbs_solver* s, const void* src, const void* x0, bool adj)
 {
     const long long n = field_len(s);
-    k_scale_source<<<voxel_grid(s), 256, 0, s->st>>>(scale_in(s), (const double2*)src, s->y64, adj ? 1 : 0);
+    k_scale_source<<<scale_grid(s), 256, 0, s->st>>>(scale_in(s), (const double2*)src, s->y64, adj ? 1 : 0);
     CUDA_TRY(cudaGetLastError());
     s->launches += x0 ? 2 : 1;
     if (x0) {
@@ -957,7 +972,7 @@ cbs_status solve_plain_32(cbs_solver* s, const void* src, void* field, const voi
         return CBS_OK;
     }
     const double ys = std::sqrt(ny2);
-    k_scale_source_32<<<g, 256, 0, s->st>>>(p, sp, s->y32, 1.0 / ys, adj ? 1 : 0);
+    k_scale_source_32<<<scale_grid(s), 256, 0, s->st>>>(p, sp, s->y32, 1.0 / ys, adj ? 1 : 0);
     CUDA_TRY(cudaGetLastError());
     s->launches += 1;
     if (x0) {
@@ -1742,7 +1757,7 @@ cbs_status scale_source(cbs_solver* s, const void* src, void* y, int adjoint)
     try {
         begin_call(s);
         const long long n = field_len(s);
-        k_scale_source<<<voxel_grid(s), 256, 0, s->st>>>(scale_in(s), (const double2*)src, (double2*)y, adjoint ? 1 : 0);
+        k_scale_source<<<scale_grid(s), 256, 0, s->st>>>(scale_in(s), (const double2*)src, (double2*)y, adjoint ? 1 : 0);
         CUDA_TRY(cudaGetLastError());
         CUDA_TRY(cudaStreamSynchronize(s->st));
         return CBS_OK;
