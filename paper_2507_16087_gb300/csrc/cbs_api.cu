@@ -803,6 +803,24 @@ bool overlap(const void* a, const void* b, size_t n)
     return p < q + n && q < p + n;
 }
 
+// The float64 applies run from the caller's buffer into the caller's buffer.  Where these share memory the input goes
+// through x64 first; a buffer off the 16-byte boundaries of the kernels' loads and stores goes through x64 / w64 (a
+// caller's double complex may lie on 8 bytes, and a copy takes any alignment).
+bool off16(const void* p) { return reinterpret_cast<uintptr_t>(p) % 16 != 0; }
+const double2* apply_in(cbs_solver* s, const void* in, const void* out)
+{
+    const size_t bytes = (size_t)s->C * s->N * sizeof(double2);
+    if (!off16(in) && !overlap(in, out, bytes)) return (const double2*)in;
+    CUDA_TRY(cudaMemcpyAsync(s->x64, in, bytes, cudaMemcpyDeviceToDevice, s->st));
+    return s->x64;
+}
+double2* apply_out(cbs_solver* s, void* out) { return off16(out) ? s->w64 : (double2*)out; }
+void copy_apply(cbs_solver* s, const double2* from, void* out)
+{
+    if (from != out)
+        CUDA_TRY(cudaMemcpyAsync(out, from, (size_t)s->C * s->N * sizeof(double2), cudaMemcpyDeviceToDevice, s->st));
+}
+
 void read_red(cbs_solver* s, double* out2)
 {
     CUDA_TRY(cudaMemcpyAsync(s->host_red, s->red, 2 * sizeof(double), cudaMemcpyDeviceToHost, s->st));
@@ -1715,13 +1733,10 @@ cbs_status green_apply(cbs_solver* s, const void* in, void* out, int adjoint)
             k_cast_32_64<<<grid_for(n), 256, 0, s->st>>>(s->w32, (double2*)out, n);
             CUDA_TRY(cudaGetLastError());
         } else {
-            // straight from the caller's buffer into the caller's buffer, unless they share memory
-            const double2* x = (const double2*)in;
-            if (overlap(in, out, n * sizeof(double2))) {
-                CUDA_TRY(cudaMemcpyAsync(s->x64, in, n * sizeof(double2), cudaMemcpyDeviceToDevice, s->st));
-                x = s->x64;
-            }
-            CUDA_TRY(launch_green<double>(s->P64, x, (double2*)out, adjoint != 0, s->st));
+            const double2* x = apply_in(s, in, out);
+            double2* w = apply_out(s, out);
+            CUDA_TRY(launch_green<double>(s->P64, x, w, adjoint != 0, s->st));
+            copy_apply(s, w, out);
         }
         CUDA_TRY(cudaStreamSynchronize(s->st));
         return CBS_OK;
@@ -1736,13 +1751,10 @@ cbs_status operator_apply(cbs_solver* s, const void* x, void* out, int adjoint)
     if (!x || !out) return set_err(s, CBS_EINVAL, "NULL argument");
     try {
         begin_call(s);
-        const long long n = field_len(s);
-        const double2* xi = (const double2*)x;
-        if (overlap(x, out, n * sizeof(double2))) {
-            CUDA_TRY(cudaMemcpyAsync(s->x64, x, n * sizeof(double2), cudaMemcpyDeviceToDevice, s->st));
-            xi = s->x64;
-        }
-        CUDA_TRY(launch_operator<double>(s->P64, xi, nullptr, (double2*)out, OP_APPLY, adjoint != 0, s->partials, s->st));
+        const double2* xi = apply_in(s, x, out);
+        double2* w = apply_out(s, out);
+        CUDA_TRY(launch_operator<double>(s->P64, xi, nullptr, w, OP_APPLY, adjoint != 0, s->partials, s->st));
+        copy_apply(s, w, out);
         CUDA_TRY(cudaStreamSynchronize(s->st));
         return CBS_OK;
     } catch (const CudaError& e) {
