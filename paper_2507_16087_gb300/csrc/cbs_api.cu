@@ -1454,6 +1454,9 @@ cbs_status solver_create(const cbs_grid* grid, double dx, double omega, const do
     s->omega = omega;
     s->opt = o;
     s->bnd = b;
+    // host tables of copies in flight: they outlive the try block, whose failure paths end in solver_destroy's
+    // synchronisation
+    TablePack pack, green_pack;
     try {
         TRACE("create: stream");
         CUDA_TRY(cudaStreamCreateWithFlags(&s->st, cudaStreamNonBlocking));
@@ -1470,7 +1473,6 @@ cbs_status solver_create(const cbs_grid* grid, double dx, double omega, const do
         const long long N = s->N;
         const int D = s->D;
         // per-axis tables (host, float64): gamma, wavenumbers, twiddles
-        TablePack pack, green_pack;  // alive until the last synchronisation below
         for (int a = 0; a < 3; ++a) {
             const int n = s->n[a];
             std::vector<double> gc(n, 0.0), gs(n, 0.0), k2(n, 0.0);
