@@ -252,6 +252,15 @@ cudaError_t launch_rows_op(const Plan<R>& P, const cplx<R>* x, const cplx<R>* y,
     }
 }
 
+// Whether the small tile of an axis is another one at all, and for float32 of fewer columns: from 1024 points it has the
+// big tile's columns, so it makes no more blocks, and its 1024-thread blocks spill (us an iteration: 2048 points 8 columns
+// 23.2 against 19.1 with the big tile, 128 columns 29.2 against 25.1, 512 columns 53.2 against 47.5; 1024 points 64 columns
+// 14.3 against 14.0, 512 columns 29.0 against 28.5).
+template <typename R> constexpr bool has_small_tile(int n)
+{
+    return sizeof(R) == 4 ? cols_small<R>(n) < cols_big<R>(n)
+                          : cols_small<R>(n) != cols_big<R>(n) || r_tile<R>(n) != r_axis<R>(n);
+}
 // whether a strided axis of N points and `columns` columns (of two transforms) takes the small tiles: float32 when the
 // big ones leave SMs without a block (64^3, 256 tiles: 20.3 us an iteration with the big ones against 20.9; 512^2, 64
 // tiles: 17.8 against 15.9), float64 when the big ones make too few warps
@@ -275,7 +284,7 @@ template <typename R, int N, int RA, int COLS, int S> cudaError_t axis2_tile(con
 template <typename R, int N, int S> cudaError_t axis2_n(const Plan<R>& P, cplx<R>* w, int adj, cudaStream_t st)
 {
     constexpr int CB = cols_big<R>(N), CS = cols_small<R>(N);
-    if constexpr (CS != CB || r_tile<R>(N) != r_axis<R>(N)) {
+    if constexpr (has_small_tile<R>(N)) {
         if (small_tiles<R, N>((long long)P.d.n0 * P.d.n2 * 3 / 2))
             return axis2_tile<R, N, r_tile<R>(N), CS, S>(P, w, adj, st);
     }
@@ -306,7 +315,7 @@ template <typename R, int N> cudaError_t last2_n(const Plan<R>& P, cplx<R>* w, i
 {
     constexpr int CB = cols_big<R>(N), CS = cols_small<R>(N);
     const long long ncol = P.d.D == 3 ? (long long)P.d.n0 * P.d.n1 : P.d.n0;
-    if constexpr (CS != CB || r_tile<R>(N) != r_axis<R>(N)) {
+    if constexpr (has_small_tile<R>(N)) {
         if (small_tiles<R, N>(ncol)) return last2_tile<R, N, r_tile<R>(N), CS>(P, w, adj, st);
     }
     return last2_tile<R, N, r_last<R>(N), CB>(P, w, adj, st);
@@ -339,7 +348,7 @@ template <typename R, int N>
 cudaError_t deriv_n(const Plan<R>& P, const cplx<R>* x, cplx<R>* w, int e, int add, int adj, cudaStream_t st)
 {
     constexpr int CB = cols_big<R>(N), CS = cols_small<R>(N);
-    if constexpr (CS != CB || r_tile<R>(N) != r_axis<R>(N)) {
+    if constexpr (has_small_tile<R>(N)) {
         if (small_tiles<R, N>(P.d.N / N)) return deriv_tile<R, N, r_tile<R>(N), CS>(P, x, w, e, add, adj, st);
     }
     return deriv_tile<R, N, r_axis<R>(N), CB>(P, x, w, e, add, adj, st);

@@ -1,6 +1,7 @@
-"""Shared memory the row kernels' launches ask for (csrc/launch.cuh), on the CPU: the launchers run against a stand-in
-for the runtime's launch call that records each launch.  A block must not take room that its mode or row length never
-touches, or fewer blocks fit on an SM than the kernel was compiled for."""
+"""Launches of the kernels of an iteration (csrc/launch.cuh), on the CPU: the launchers run against a stand-in for the
+runtime's launch call that records each launch.  A row block must not take shared memory that its mode or row length
+never touches, or fewer blocks fit on an SM than the kernel was compiled for; a strided axis takes its small tile only
+where that makes more blocks."""
 import ctypes
 import os
 import shutil
@@ -21,6 +22,7 @@ extern "C" cudaError_t cudaLaunchKernelExC(const cudaLaunchConfig_t* c, const vo
 extern "C" cudaError_t cudaFuncSetAttribute(const void*, cudaFuncAttribute, int) { return cudaSuccess; }
 #include "launch.cuh"
 using namespace cbs;
+using P32 = Plan<float>;
 
 template <typename R, int N> int run(int D, int n1, int n2, int mode, int* o)
 {
@@ -36,6 +38,27 @@ template <typename R, int N> int run(int D, int n1, int n2, int mode, int* o)
     o[5] = (tiny ? B::ML : A::ML) * (int)sizeof(R);        // a medium row
     o[6] = g_threads / (tiny ? B::T : A::T);               // units
     return (int)e;
+}
+// whether a float32 axis of N points and `columns` columns takes the small tile, and the blocks either tile makes
+template <int N> int tiles(long long columns, int* o)
+{
+    P32 P{};
+    P.d.D = 2; P.d.n0 = (int)columns; P.d.n1 = N; P.d.n2 = 1; P.d.N = columns * N;
+    const cudaError_t e = last2_n<float, N>(P, nullptr, 0, nullptr);
+    o[0] = g_blocks; o[1] = g_threads;
+    o[2] = (int)((columns + cols_big<float>(N) - 1) / cols_big<float>(N));
+    o[3] = N / r_axis<float>(N) * cols_big<float>(N);
+    return (int)e;
+}
+extern "C" int last_launch(int n, long long columns, int* o)
+{
+    switch (n) {
+    case 64: return tiles<64>(columns, o);
+    case 512: return tiles<512>(columns, o);
+    case 1024: return tiles<1024>(columns, o);
+    case 2048: return tiles<2048>(columns, o);
+    }
+    return -1;
 }
 extern "C" int row_launch(int f64, int D, int n0, int n1, int n2, int mode, int* o)
 {
@@ -61,6 +84,7 @@ def lib():
                            "-o", so])
     L = ctypes.CDLL(so)
     L.row_launch.argtypes = [ctypes.c_int] * 6 + [ctypes.c_void_p]
+    L.last_launch.argtypes = [ctypes.c_int, ctypes.c_longlong, ctypes.c_void_p]
     return L
 
 
@@ -92,3 +116,12 @@ def test_a_launch_asks_for_the_buffers_its_mode_uses(lib, f64, grid, mode):
     # y may have a buffer of its own in the updates, for rows whose y is staged; the barriers take up to 32 bytes
     own_y = g["units"] * g["row"] if mode in (FUSED, FUSED_NORM, INV) and not (grid[0] >= 1024 and not f64) else 0
     assert g["smem"] in (least, least + 32, least + own_y + 32)
+
+
+@pytest.mark.parametrize("n", [64, 512, 1024, 2048])
+@pytest.mark.parametrize("columns", [8, 48, 128, 512, 1024, 2048])
+def test_a_small_tile_is_taken_for_more_blocks(lib, n, columns):
+    o = (ctypes.c_int * 4)()
+    assert lib.last_launch(n, columns, o) == 0
+    blocks, threads, big_blocks, big_threads = o
+    assert (blocks, threads) == (big_blocks, big_threads) or (blocks > big_blocks and threads <= big_threads)
