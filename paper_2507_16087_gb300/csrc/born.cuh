@@ -143,18 +143,18 @@ __device__ __forceinline__ cplx<R> born_B(const Medium<R>& M, const RowB<R>& rb,
 // the one before it is complete and visible; only what the direct predecessor writes has to wait.
 // The trigger comes before a block's last stores: the next kernel's blocks then find free SMs and start evenly.  Given
 // right after the wait it packs them onto the SMs that finish first (64^3 23.6 against 20.9 us an iteration, 512^2 19.3
-// against 15.7, 512^3 8.7 against 7.5 ms); only a float32 grid of at most one block an SM gains (128^2 8.1 against 9.4
-// us; float64 kernels are not launched this way, see kDependent in launch.cuh).
+// against 15.7, 512^3 8.7 against 7.5 ms); only where neither kernel fills the SMs does the earlier start gain (early_next in
+// launch.cuh; float64 kernels are not launched this way, see kDependent there).
 __device__ __forceinline__ void grid_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void grid_trigger() { asm volatile("griddepcontrol.launch_dependents;"); }
 constexpr int kSMs = 152;
-template <typename R> __device__ __forceinline__ void grid_trigger_small()  // (predicated: a branch here splits the loads that follow)
+template <typename R> __device__ __forceinline__ void grid_trigger_if(int early)  // (predicated: a branch here splits the loads that follow)
 {
     if constexpr (sizeof(R) == 4)
         asm volatile(
             "{\n\t.reg .pred p;\n\t"
-            "setp.le.u32 p, %0, %1;\n\t"
-            "@p griddepcontrol.launch_dependents;\n\t}" ::"r"(gridDim.x), "n"(kSMs));
+            "setp.ne.s32 p, %0, 0;\n\t"
+            "@p griddepcontrol.launch_dependents;\n\t}" ::"r"(early));
 }
 
 template <int T> struct RowSync {
@@ -329,7 +329,7 @@ template <bool PAIR, typename R> __device__ __forceinline__ cplx<R> voxel_B(cons
 template <typename R, int NX, int RX, int MODE>
 __global__ void __launch_bounds__(RowCfg<R, NX, RX>::MAXT, RowCfg<R, NX, RX>::MINB)
 k_rows(Dims d, Medium<R> M, Symbol<R> Sy, cplx<R>* __restrict__ x, const cplx<R>* __restrict__ y,
-       cplx<R>* __restrict__ w, const cplx<R>* __restrict__ tw, int npair, int nsingle, int ysep, int adj, R nu,
+       cplx<R>* __restrict__ w, const cplx<R>* __restrict__ tw, int npair, int nsingle, int ysep, int early, int adj, R nu,
        double* __restrict__ partials, int* err)
 {
     using CT = cplx<R>;
@@ -383,7 +383,7 @@ k_rows(Dims d, Medium<R> M, Symbol<R> Sy, cplx<R>* __restrict__ x, const cplx<R>
     // w goes first, the transform waits for nothing else (512^3 3.54 against 3.64 ms, 2048^2 154 against 161 us).
     auto w_in = [&]() {
         grid_wait();
-        grid_trigger_small<R>();
+        grid_trigger_if<R>(early);
         if constexpr (UPDATE) rows_in(ws, w + (long long)cs * d.N + v0, SL, FB, bar);
     };
     auto y_in = [&](uint64_t* on) {
@@ -598,7 +598,7 @@ __device__ __forceinline__ void col_store(CT* p, long long st, const CT (&v)[RA]
 // thread (the column and the one half the columns further on).
 template <typename R, int NA, int RA, int COLS, int S>
 __global__ void __launch_bounds__(PairCfg<R, NA, RA, COLS>::THREADS, PairCfg<R, NA, RA, COLS>::MINB)
-k_axis2(Dims d, cplx<R>* __restrict__ w, const cplx<R>* __restrict__ tw, const cplx<R>* __restrict__ tab, int npair)
+k_axis2(Dims d, cplx<R>* __restrict__ w, const cplx<R>* __restrict__ tw, const cplx<R>* __restrict__ tab, int npair, int early)
 {
     using CT = cplx<R>;
     using Cfg = PairCfg<R, NA, RA, COLS>;
@@ -621,7 +621,7 @@ k_axis2(Dims d, cplx<R>* __restrict__ w, const cplx<R>* __restrict__ tw, const c
     const long long st = (long long)T * d.n0;
     CT v[2][RA];
     grid_wait();
-    grid_trigger_small<R>();
+    grid_trigger_if<R>(early);
     col_load<NA, RA, 0>(v[0], a, st);
     if (S < 0 || !pair) {
         col_load<NA, RA, 0>(v[1], b, st);
@@ -647,7 +647,7 @@ k_axis2(Dims d, cplx<R>* __restrict__ w, const cplx<R>* __restrict__ tw, const c
 // ms at 512^3 (79 and 632 us at HBM rate); holding all four components it took 40.5 us, 334 us and 3.24 ms.
 template <typename R, int NL, int RL, int COLS>
 __global__ void __launch_bounds__(PairCfg<R, NL, RL, COLS>::THREADS, PairCfg<R, NL, RL, COLS>::MINB)
-k_last2(Dims d, Symbol<R> Sy, cplx<R>* __restrict__ w, const cplx<R>* __restrict__ tw)
+k_last2(Dims d, Symbol<R> Sy, cplx<R>* __restrict__ w, const cplx<R>* __restrict__ tw, int early)
 {
     using CT = cplx<R>;
     using Cfg = PairCfg<R, NL, RL, COLS>;
@@ -665,7 +665,7 @@ k_last2(Dims d, Symbol<R> Sy, cplx<R>* __restrict__ w, const cplx<R>* __restrict
     const long long st = (long long)T * ncol;
     CT v[2][RL];
     grid_wait();
-    if (sizeof(R) == 4 && gridDim.x <= kSMs) grid_trigger();  // (a branch, not the predicated form: 137 against 151 us at 256^3)
+    if (sizeof(R) == 4 && early) grid_trigger();  // (a branch, not the predicated form: 137 against 151 us at 256^3)
     col_load<NL, RL, 0>(v[0], a, st);
     col_load<NL, RL, 0>(v[1], b, st);
     R k2c = Sy.c3.x;
@@ -723,7 +723,7 @@ k_deriv2(Dims d, LOp<R> L, const cplx<R>* __restrict__ x, cplx<R>* __restrict__ 
     const long long st = (long long)T * astride;
     CT v[2][RA];
     grid_wait();
-    grid_trigger_small<R>();
+    grid_trigger_if<R>(gridDim.x <= kSMs);
     col_load<N, RA, 0>(v[0], x + oa, st);
     col_load<N, RA, 0>(v[1], x + ob, st);
     fft_run_multi<N, RA, 2, -1, Cfg::PADC>(v, sm + col, COLS, Cfg::FSTRIDE, t, tw, BlockSync());
@@ -790,7 +790,7 @@ k_rows_op(Dims d, Medium<R> M, LOp<R> L, const cplx<R>* __restrict__ x, const cp
     const RowB<R> rb = row_B(M, d.D, c, i1, i2, vbase);
     CT v[RX];
     grid_wait();
-    grid_trigger_small<R>();
+    grid_trigger_if<R>(gridDim.x <= kSMs);
     if (pair) {
         TwCache<NX, RX, CT> tc;
         tw_load<NX, RX, T>(tc, t, tw);

@@ -120,12 +120,13 @@ template <typename R, int N, int RX> inline int rows_units_n(const Dims& d)
 }
 // whether the row kernels take r_rows_tile values a thread on this grid: float64 where r_rows leaves too few warps,
 // float32 512-point rows where all of them are on the SMs at once (512^2: 14.5 against 16.1 us an iteration)
-template <typename R, int N> inline bool rows_tiny(const Dims& d)
+template <typename R> inline bool rows_tiny(int n, const Dims& d)
 {
-    if (r_rows_tile<R>(N) >= r_rows<R>(N)) return false;
+    if (r_rows_tile<R>(n) >= r_rows<R>(n)) return false;
     const long long values = (long long)(d.D + 1) * d.N;
-    return sizeof(R) == 8 ? few_warps<R>(values, r_rows<R>(N)) : values / r_rows<R>(N) <= 512LL * kSMs;
+    return sizeof(R) == 8 ? few_warps<R>(values, r_rows<R>(n)) : values / r_rows<R>(n) <= 512LL * kSMs;
 }
+template <typename R, int N> inline bool rows_tiny(const Dims& d) { return rows_tiny<R>(N, d); }
 
 struct RowGrid {
     int units, npair, nsingle, blocks;
@@ -140,6 +141,51 @@ template <typename R, int N> inline RowGrid row_grid(const Dims& d)
     g.blocks = g.npair + (d.D - 1) * g.nsingle;
     return g;
 }
+
+// Whether the small tile of an axis is another one at all, and for float32 of fewer columns: from 1024 points it has the
+// big tile's columns, so it makes no more blocks, and its 1024-thread blocks spill (us an iteration: 2048 points 8 columns
+// 23.2 against 19.1 with the big tile, 128 columns 29.2 against 25.1, 512 columns 53.2 against 47.5; 1024 points 64 columns
+// 14.3 against 14.0, 512 columns 29.0 against 28.5).
+template <typename R> constexpr bool has_small_tile(int n)
+{
+    return sizeof(R) == 4 ? cols_small<R>(n) < cols_big<R>(n)
+                          : cols_small<R>(n) != cols_big<R>(n) || r_tile<R>(n) != r_axis<R>(n);
+}
+// whether a strided axis of N points and `columns` columns (of two transforms) takes the small tiles: float32 when the
+// big ones leave SMs without a block (64^3, 256 tiles: 20.3 us an iteration with the big ones against 20.9; 512^2, 64
+// tiles: 17.8 against 15.9), float64 when the big ones make too few warps
+template <typename R> inline bool small_tiles(int n, long long columns)
+{
+    if (!has_small_tile<R>(n)) return false;
+    if (sizeof(R) == 8) return few_warps<R>(columns * n, r_axis<R>(n));
+    return (columns + cols_big<R>(n) - 1) / cols_big<R>(n) < kSMs;
+}
+
+// Whether a float32 kernel of `blocks` blocks lets the next one start right after its own wait (see grid_wait): with at most
+// a block an SM itself, and where the next kernel's blocks, packed onto the SMs with room, don't crowd them: one warp an SM of
+// a strided axis or six of the row kernel.  us an iteration, early / late.  Rows before a strided axis: 24 x 2048 (128 warps)
+// 12.0 / 15.2, 48 x 1024 (128) 10.8 / 12.8, 96 x 1024 (256) 13.3 / 12.4, 96 x 2048 (512) 18.8 / 15.6.  Last axis before rows:
+// 128^2 (192 warps) 7.4 / 8.4, 256^2 (384) 9.0 / 10.1, 96 x 512 (576) 10.1 / 10.9, 512 x 128 (768) 9.8 / 10.3, 192 x 512
+// (1152) 13.3 / 11.3, 256 x 512 (1536) 12.1 / 10.0.
+template <typename R> inline int early_next(const Dims& d, long long blocks, bool rows_next, int n, long long columns)
+{
+    if (sizeof(R) != 4 || blocks > kSMs) return 0;
+    if (rows_next) {
+        const int r = rows_tiny<R>(d.n0, d) ? r_rows_tile<R>(d.n0) : r_rows<R>(d.n0);
+        return (d.D + 1) * d.N / r <= 6 * 32 * kSMs;
+    }
+    const int r = small_tiles<R>(n, columns) ? r_tile<R>(n) : r_axis<R>(n);
+    return columns * (n / r) <= 32 * kSMs;
+}
+// columns (of two transforms) of the y axis of a 3D field and of the last axis
+inline long long axis_columns(const Dims& d) { return (long long)d.n0 * d.n2 * 3 / 2; }
+inline long long last_columns(const Dims& d) { return d.D == 3 ? (long long)d.n0 * d.n1 : d.n0; }
+template <typename R> inline int early_axis(const Dims& d, long long blocks) { return early_next<R>(d, blocks, false, d.n1, axis_columns(d)); }
+template <typename R> inline int early_last(const Dims& d, long long blocks)
+{
+    return early_next<R>(d, blocks, false, d.D == 3 ? d.n2 : d.n1, last_columns(d));
+}
+template <typename R> inline int early_rows(const Dims& d, long long blocks) { return early_next<R>(d, blocks, true, 0, 0); }
 
 // blocks of the row kernels (= norm partials of one iteration)
 template <typename R> inline int rows_blocks(const Plan<R>& P)
@@ -174,7 +220,8 @@ cudaError_t rows_nm(const Plan<R>& P, cplx<R>* x, const cplx<R>* y, cplx<R>* w, 
     const int ysep = kOwnY && g.blocks <= 4 * kWaveBlocks ? 1 : 0;
     // the modes that start a chain follow other work (x and y may have just been written)
     return launch(kern, g.blocks, g.units * Cfg::T, Cfg::smem(g.units, MODE, ysep != 0), st,
-                  kDependent<R> && MODE != ROWS_FWD && MODE != ROWS_COPY, P.d, P.M, P.Sy[adj ? 1 : 0], x, y, w, P.tw[0], g.npair, g.nsingle, ysep, adj, nu, partials, P.err);
+                  kDependent<R> && MODE != ROWS_FWD && MODE != ROWS_COPY, P.d, P.M, P.Sy[adj ? 1 : 0], x, y, w, P.tw[0], g.npair, g.nsingle, ysep,
+                  P.d.D == 3 ? early_axis<R>(P.d, g.blocks) : early_last<R>(P.d, g.blocks), adj, nu, partials, P.err);
 }
 
 template <typename R, int N, int RX>
@@ -252,24 +299,6 @@ cudaError_t launch_rows_op(const Plan<R>& P, const cplx<R>* x, const cplx<R>* y,
     }
 }
 
-// Whether the small tile of an axis is another one at all, and for float32 of fewer columns: from 1024 points it has the
-// big tile's columns, so it makes no more blocks, and its 1024-thread blocks spill (us an iteration: 2048 points 8 columns
-// 23.2 against 19.1 with the big tile, 128 columns 29.2 against 25.1, 512 columns 53.2 against 47.5; 1024 points 64 columns
-// 14.3 against 14.0, 512 columns 29.0 against 28.5).
-template <typename R> constexpr bool has_small_tile(int n)
-{
-    return sizeof(R) == 4 ? cols_small<R>(n) < cols_big<R>(n)
-                          : cols_small<R>(n) != cols_big<R>(n) || r_tile<R>(n) != r_axis<R>(n);
-}
-// whether a strided axis of N points and `columns` columns (of two transforms) takes the small tiles: float32 when the
-// big ones leave SMs without a block (64^3, 256 tiles: 20.3 us an iteration with the big ones against 20.9; 512^2, 64
-// tiles: 17.8 against 15.9), float64 when the big ones make too few warps
-template <typename R, int N> inline bool small_tiles(long long columns)
-{
-    if (sizeof(R) == 8) return few_warps<R>(columns * N, r_axis<R>(N));
-    return (columns + cols_big<R>(N) - 1) / cols_big<R>(N) < kSMs;
-}
-
 template <typename R, int N, int RA, int COLS, int S> cudaError_t axis2_tile(const Plan<R>& P, cplx<R>* w, int adj, cudaStream_t st)
 {
     using Cfg = PairCfg<R, N, RA, COLS>;
@@ -277,15 +306,16 @@ template <typename R, int N, int RA, int COLS, int S> cudaError_t axis2_tile(con
     static const cudaError_t attr = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)Cfg::SMEM);
     if (attr != cudaSuccess) return attr;
     const int ncol = P.d.n0 * P.d.n2;
-    const int npair = (ncol + COLS - 1) / COLS, nz = (ncol / 2 + COLS - 1) / COLS;
+    const int npair = (ncol + COLS - 1) / COLS, blocks = npair + (ncol / 2 + COLS - 1) / COLS;
     const Symbol<R>& Sy = P.Sy[adj ? 1 : 0];
-    return launch(kern, npair + nz, Cfg::THREADS, Cfg::SMEM, st, kDependent<R>, P.d, w, P.tw[1], S < 0 ? Sy.tm[1] : Sy.td[1], npair);
+    return launch(kern, blocks, Cfg::THREADS, Cfg::SMEM, st, kDependent<R>, P.d, w, P.tw[1], S < 0 ? Sy.tm[1] : Sy.td[1], npair,
+                  S < 0 ? early_last<R>(P.d, blocks) : early_rows<R>(P.d, blocks));
 }
 template <typename R, int N, int S> cudaError_t axis2_n(const Plan<R>& P, cplx<R>* w, int adj, cudaStream_t st)
 {
     constexpr int CB = cols_big<R>(N), CS = cols_small<R>(N);
     if constexpr (has_small_tile<R>(N)) {
-        if (small_tiles<R, N>((long long)P.d.n0 * P.d.n2 * 3 / 2))
+        if (small_tiles<R>(N, axis_columns(P.d)))
             return axis2_tile<R, N, r_tile<R>(N), CS, S>(P, w, adj, st);
     }
     return axis2_tile<R, N, r_axis<R>(N), CB, S>(P, w, adj, st);
@@ -308,15 +338,15 @@ template <typename R, int N, int RL, int COLS> cudaError_t last2_tile(const Plan
     auto kern = k_last2<R, N, RL, COLS>;
     static const cudaError_t attr = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)Cfg::SMEM);
     if (attr != cudaSuccess) return attr;
-    const long long ncol = P.d.D == 3 ? (long long)P.d.n0 * P.d.n1 : P.d.n0;
-    return launch(kern, (ncol + COLS - 1) / COLS, Cfg::THREADS, Cfg::SMEM, st, kDependent<R>, P.d, P.Sy[adj ? 1 : 0], w, P.tw[P.d.D - 1]);
+    const long long blocks = (last_columns(P.d) + COLS - 1) / COLS;
+    return launch(kern, blocks, Cfg::THREADS, Cfg::SMEM, st, kDependent<R>, P.d, P.Sy[adj ? 1 : 0], w, P.tw[P.d.D - 1],
+                  P.d.D == 3 ? early_axis<R>(P.d, blocks) : early_rows<R>(P.d, blocks));
 }
 template <typename R, int N> cudaError_t last2_n(const Plan<R>& P, cplx<R>* w, int adj, cudaStream_t st)
 {
     constexpr int CB = cols_big<R>(N), CS = cols_small<R>(N);
-    const long long ncol = P.d.D == 3 ? (long long)P.d.n0 * P.d.n1 : P.d.n0;
     if constexpr (has_small_tile<R>(N)) {
-        if (small_tiles<R, N>(ncol)) return last2_tile<R, N, r_tile<R>(N), CS>(P, w, adj, st);
+        if (small_tiles<R>(N, last_columns(P.d))) return last2_tile<R, N, r_tile<R>(N), CS>(P, w, adj, st);
     }
     return last2_tile<R, N, r_last<R>(N), CB>(P, w, adj, st);
 }
@@ -349,7 +379,7 @@ cudaError_t deriv_n(const Plan<R>& P, const cplx<R>* x, cplx<R>* w, int e, int a
 {
     constexpr int CB = cols_big<R>(N), CS = cols_small<R>(N);
     if constexpr (has_small_tile<R>(N)) {
-        if (small_tiles<R, N>(P.d.N / N)) return deriv_tile<R, N, r_tile<R>(N), CS>(P, x, w, e, add, adj, st);
+        if (small_tiles<R>(N, P.d.N / N)) return deriv_tile<R, N, r_tile<R>(N), CS>(P, x, w, e, add, adj, st);
     }
     return deriv_tile<R, N, r_axis<R>(N), CB>(P, x, w, e, add, adj, st);
 }

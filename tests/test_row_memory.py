@@ -16,9 +16,13 @@ FWD, FUSED, FUSED_NORM, INV, COPY, GREEN = range(6)  # RowsMode
 
 SRC = r'''
 #include <cuda_runtime.h>
-static int g_threads, g_smem, g_blocks;
-extern "C" cudaError_t cudaLaunchKernelExC(const cudaLaunchConfig_t* c, const void*, void**)
-{ g_threads = c->blockDim.x; g_smem = (int)c->dynamicSmemBytes; g_blocks = c->gridDim.x; return cudaSuccess; }
+static int g_threads, g_smem, g_blocks, g_early, g_early_arg;
+extern "C" cudaError_t cudaLaunchKernelExC(const cudaLaunchConfig_t* c, const void*, void** args)
+{
+    g_threads = c->blockDim.x; g_smem = (int)c->dynamicSmemBytes; g_blocks = c->gridDim.x;
+    if (g_early_arg > 0) g_early = *(const int*)args[g_early_arg];
+    return cudaSuccess;
+}
 extern "C" cudaError_t cudaFuncSetAttribute(const void*, cudaFuncAttribute, int) { return cudaSuccess; }
 #include "launch.cuh"
 using namespace cbs;
@@ -49,6 +53,31 @@ template <int N> int tiles(long long columns, int* o)
     o[2] = (int)((columns + cols_big<float>(N) - 1) / cols_big<float>(N));
     o[3] = N / r_axis<float>(N) * cols_big<float>(N);
     return (int)e;
+}
+// the early flags of the row and the last-axis kernel of a 2D grid (arguments 10 of k_rows, 4 of k_last2)
+template <int N0, int N1> int early2(int* o)
+{
+    P32 P{};
+    P.d.D = 2; P.d.n0 = N0; P.d.n1 = N1; P.d.n2 = 1; P.d.N = (long long)N0 * N1;
+    g_early_arg = 10;
+    cudaError_t e = rows_n<float, N0>(P, nullptr, nullptr, nullptr, ROWS_FUSED, 0, 0.0f, nullptr, nullptr);
+    o[0] = g_early;
+    g_early_arg = 4;
+    if (e == cudaSuccess) e = last2_n<float, N1>(P, nullptr, 0, nullptr);
+    o[1] = g_early;
+    g_early_arg = 0;
+    return (int)e;
+}
+extern "C" int early(int k, int* o)
+{
+    switch (k) {
+    case 0: return early2<2048, 24>(o);
+    case 1: return early2<2048, 96>(o);
+    case 2: return early2<512, 192>(o);
+    case 3: return early2<128, 128>(o);
+    case 4: return early2<1024, 1024>(o);
+    }
+    return -1;
 }
 extern "C" int last_launch(int n, long long columns, int* o)
 {
@@ -85,6 +114,7 @@ def lib():
     L = ctypes.CDLL(so)
     L.row_launch.argtypes = [ctypes.c_int] * 6 + [ctypes.c_void_p]
     L.last_launch.argtypes = [ctypes.c_int, ctypes.c_longlong, ctypes.c_void_p]
+    L.early.argtypes = [ctypes.c_int, ctypes.c_void_p]
     return L
 
 
@@ -125,3 +155,13 @@ def test_a_small_tile_is_taken_for_more_blocks(lib, n, columns):
     assert lib.last_launch(n, columns, o) == 0
     blocks, threads, big_blocks, big_threads = o
     assert (blocks, threads) == (big_blocks, big_threads) or (blocks > big_blocks and threads <= big_threads)
+
+
+# 2048 x 24: 36 row blocks before 128 warps, 128 last-axis blocks before 288; 2048 x 96: 144 row blocks before 512 warps, 512
+# last-axis blocks; 512 x 192: the last axis before 1152 warps of rows; 128^2: 192 row blocks, the last axis before 192
+# warps; 1024^2: more than a block an SM everywhere
+@pytest.mark.parametrize("case,rows,last", [(0, 1, 1), (1, 0, 0), (2, 0, 0), (3, 0, 1), (4, 0, 0)])
+def test_the_next_kernel_starts_early_where_it_does_not_crowd(lib, case, rows, last):
+    o = (ctypes.c_int * 2)()
+    assert lib.early(case, o) == 0
+    assert list(o) == [rows, last]
