@@ -18,7 +18,8 @@
 //   * Pu v_eta is added in real space (v = B x + y is there anyway), and td_eta p splits off the pressure at
 //     the inverse transform of axis eta.
 // The fields carried between the kernels are q (partial sum, later the pressure) in component slot D of w and the
-// velocity components not yet merged (later the split-off gradients) in their own slots; slot 0 is never used:
+// velocity components not yet merged (later the split-off gradients) in their own slots; slot 0 is used by rows apart only
+// (k_rows):
 //     rows     update of iteration k, then B x + y and the forward x transform: p and u_x merge into q
 //     axis2 +  forward y transform (3D): u_y merges into q               3 fields in, 2 out
 //     last2    forward transform of the last axis, the scalar solve, inverse transform: 2 fields in, 2 out
@@ -268,7 +269,9 @@ __device__ __forceinline__ void fence_proxy_async_smem() { asm volatile("fence.p
 // exchange runs in the staged w row and the rows that share a shared-memory phase lie on different banks.
 // y lands in w's rows once the inverse transform has been read out of them (ysep = 0: two field buffers a block,
 // more blocks an SM) or in a buffer of its own, issued at the start (ysep = 1: small grids, where a block's
-// chain of waits is the time); rows of 1024 and more float32 points have no such buffer (YREG).  The two modes without B (ROWS_COPY, ROWS_GREEN) load straight from global memory.
+// chain of waits is the time); rows of 1024 and more float32 points have no such buffer (YREG).
+// APART (2D): every block holds one unit, u_x's too.  Its row keeps its own slot 0; k_last2's MERGE_X merges and splits it,
+// a factor a column there, so that no block waits for or reads another's row.  The two modes without B (ROWS_COPY, ROWS_GREEN) load straight from global memory.
 template <typename R, int NX, int RX> struct RowCfg {
     static constexpr int T = NX / RX;
     static constexpr int SL = RowPad<cplx<R>, NX, T>::SL;        // row pitch of the field buffers (values)
@@ -299,6 +302,13 @@ template <typename R, int NX, int RX> struct RowCfg {
         if (mode == ROWS_COPY || mode == ROWS_GREEN) return field;
         return field * (own_y(mode) && ysep ? 3 : 2) + (size_t)U / 2 * 3 * ML * sizeof(R) + 32;
     }
+    // of a block of one unit of its own (APART): its field buffers, two medium rows, the barriers
+    __host__ __device__ static constexpr size_t smem_apart(int mode)
+    {
+        const size_t field = SL * sizeof(cplx<R>);
+        if (mode == ROWS_COPY || mode == ROWS_GREEN) return field;
+        return field * (own_y(mode) ? 3 : 2) + (size_t)2 * ML * sizeof(R) + 32;
+    }
 };
 
 // B = 1 - v from a voxel's medium values, m0 = rs_c (velocity, m1 = 0) or kp (pressure, m1 = et):
@@ -326,7 +336,7 @@ template <bool PAIR, typename R> __device__ __forceinline__ cplx<R> voxel_B(cons
 // Bound by HBM where w does not fit in L2 (256^3: 402 us, 164 B/voxel at 6.8 TB/s; 512^3: 3.56 ms at 6.2 TB/s), by latency
 // where it does (128^3: 55 us at 61 % of DRAM throughput, 26 warps an SM; stalls first on the staged copies).  The kernels it
 // replaced, one per component: 60.9 us, 438 us, 3.94 ms.
-template <typename R, int NX, int RX, int MODE>
+template <typename R, int NX, int RX, int MODE, bool APART = false>
 __global__ void __launch_bounds__(RowCfg<R, NX, RX>::MAXT, RowCfg<R, NX, RX>::MINB)
 k_rows(Dims d, Medium<R> M, Symbol<R> Sy, cplx<R>* __restrict__ x, const cplx<R>* __restrict__ y,
        cplx<R>* __restrict__ w, const cplx<R>* __restrict__ tw, int npair, int nsingle, int ysep, int early, int adj, R nu,
@@ -343,24 +353,24 @@ k_rows(Dims d, Medium<R> M, Symbol<R> Sy, cplx<R>* __restrict__ x, const cplx<R>
     constexpr bool YREG = UPDATE && RowCfg<R, NX, RX>::YREG;
     constexpr bool NORM = MODE == ROWS_FUSED_NORM || MODE == ROWS_INV;
     extern __shared__ __align__(128) unsigned char smraw[];
-    const int U = blockDim.x / T, H = U >> 1;
+    const int U = APART ? 1 : blockDim.x / T, H = U >> 1;
     const int E = U * SL;
     CT* xs = reinterpret_cast<CT*>(smraw);
     CT* ws = HAS_B ? xs + E : xs;
     const bool yown = Cfg::own_y(MODE) && ysep != 0;
     CT* ys = yown ? ws + E : ws;
     R* ms = reinterpret_cast<R*>(ws + (yown ? 2 * E : E));
-    uint64_t* bar = reinterpret_cast<uint64_t*>(ms + 3 * H * ML);
-    const int lu = threadIdx.x / T, t = threadIdx.x % T;
+    uint64_t* bar = reinterpret_cast<uint64_t*>(ms + (APART ? 2 : 3 * H) * ML);
+    const int lu = APART ? 0 : threadIdx.x / T, t = APART ? threadIdx.x : threadIdx.x % T;
     const long long rpc = d.N / NX;  // rows per component
-    const bool pair = (int)blockIdx.x < npair;
+    const bool pair = !APART && (int)blockIdx.x < npair;
     const int per = pair ? H : U;
     int c, b = blockIdx.x;
     if (pair) {
         c = d.D;
     } else {
         b -= npair;
-        c = 1 + b / nsingle;
+        c = (APART ? 0 : 1) + b / nsingle;
         b = b % nsingle;
     }
     const long long row0 = (long long)b * per;
@@ -369,7 +379,8 @@ k_rows(Dims d, Medium<R> M, Symbol<R> Sy, cplx<R>* __restrict__ x, const cplx<R>
     const int lrow = isx ? lu - H : lu;
     if (isx) c = 0;
     const bool valid = lrow < nrow;
-    const bool pres = pair && !isx;
+    const bool pres = APART ? c == d.D : pair && !isx;
+    const bool two_medium = pair || (APART && pres);  // et beside kp
     constexpr int nbar = UPDATE ? (YREG ? 2 : 3) : 1;
     const long long v0 = row0 * NX;  // first voxel of the block's rows
     const int cs = pair ? d.D : c;   // component (slot) of the block's first array
@@ -393,13 +404,14 @@ k_rows(Dims d, Medium<R> M, Symbol<R> Sy, cplx<R>* __restrict__ x, const cplx<R>
     if constexpr (HAS_B) {
         if (threadIdx.x == 0) {
             const uint32_t fb = (uint32_t)nrow * FB, mb = (uint32_t)nrow * MB, two = pair ? 2u : 1u;
+            const uint32_t meds = pair ? 3u : (two_medium ? 2u : 1u);
             for (int k = 0; k < nbar; ++k) mbar_init(bar + k, 1);
             if constexpr (UPDATE) {
                 mbar_expect_tx(bar, fb);
-                mbar_expect_tx(bar + 1, two * fb + (pair ? 3u : 1u) * mb);
+                mbar_expect_tx(bar + 1, two * fb + meds * mb);
                 if constexpr (!YREG) mbar_expect_tx(bar + 2, two * fb);
             } else {
-                mbar_expect_tx(bar, 2u * two * fb + (pair ? 3u : 1u) * mb);
+                mbar_expect_tx(bar, 2u * two * fb + meds * mb);
             }
         }
         __syncthreads();
@@ -411,8 +423,11 @@ k_rows(Dims d, Medium<R> M, Symbol<R> Sy, cplx<R>* __restrict__ x, const cplx<R>
             rows_in(ms, M.kp + v0, ML, MB, bx);
             rows_in(ms + H * ML, M.et + v0, ML, MB, bx);
             rows_in(ms + 2 * H * ML, M.rs[0] + v0, ML, MB, bx);
+        } else if (APART && pres) {
+            rows_in(ms, M.kp + v0, ML, MB, bx);
+            rows_in(ms + ML, M.et + v0, ML, MB, bx);
         } else {
-            rows_in(ms, (c == 1 ? M.rs[1] : M.rs[2]) + v0, ML, MB, bx);
+            rows_in(ms, (APART && c == 0 ? M.rs[0] : (c == 1 ? M.rs[1] : M.rs[2])) + v0, ML, MB, bx);
         }
         if (!UPDATE || yown) y_in(UPDATE ? bar + 2 : bar);
     }
@@ -434,7 +449,7 @@ k_rows(Dims d, Medium<R> M, Symbol<R> Sy, cplx<R>* __restrict__ x, const cplx<R>
     const CT* xr = xs + lu * SL + t;
     const CT* yr = ys + lu * SL + t;
     const R* m0r = ms + (isx ? 2 * H + lrow : lrow) * ML + t;
-    const R* m1r = ms + (H + lrow) * ML + t;
+    const R* m1r = ms + ((APART ? 1 : H) + lrow) * ML + t;
     UnitB<R> ub{};
     const R* g0 = nullptr;
     R grest = (R)0;
@@ -506,7 +521,7 @@ k_rows(Dims d, Medium<R> M, Symbol<R> Sy, cplx<R>* __restrict__ x, const cplx<R>
                 if constexpr (HAS_FWD) v[s] = cfma(bv, xn, yv);
             }
         };
-        if (pair) update(std::true_type());
+        if (two_medium) update(std::true_type());
         else update(std::false_type());
         if constexpr (NORM) {
             if (!valid) { s0 = (R)0; s1 = (R)0; }
@@ -517,7 +532,7 @@ k_rows(Dims d, Medium<R> M, Symbol<R> Sy, cplx<R>* __restrict__ x, const cplx<R>
 #pragma unroll
         for (int s = 0; s < RX; ++s) {
             const int o = T * slot_q<NX, RX, 0>(s);
-            v[s] = cfma(pair ? B_at(o, std::true_type()) : B_at(o, std::false_type()), xr[o], yr[o]);
+            v[s] = cfma(two_medium ? B_at(o, std::true_type()) : B_at(o, std::false_type()), xr[o], yr[o]);
         }
     } else if constexpr (MODE == ROWS_COPY) {
 #pragma unroll
@@ -642,10 +657,11 @@ k_axis2(Dims d, cplx<R>* __restrict__ w, const cplx<R>* __restrict__ tw, const c
 }
 
 // Last axis: forward transforms of (q, u_last), b = q + tm u_last, p = cs b / (|k|^2 + c3), inverse transforms of p
-// and td p.  grid: ceil(n0 n1 / COLS) (3D) or ceil(n0 / COLS) (2D).
+// and td p.  grid: ceil(n0 n1 / COLS) (3D) or ceil(n0 / COLS) (2D).  MERGE_X (2D, rows apart): u_x comes in slot 0 and merges
+// here, td_x p leaves there.
 // Bound on chip, by exchanges, barriers and the first loads of a wave: 22 us at 128^3 (6 at L2 rate), 129 us at 256^3 and 1.45
 // ms at 512^3 (79 and 632 us at HBM rate); holding all four components it took 40.5 us, 334 us and 3.24 ms.
-template <typename R, int NL, int RL, int COLS>
+template <typename R, int NL, int RL, int COLS, bool MERGE_X = false>
 __global__ void __launch_bounds__(PairCfg<R, NL, RL, COLS>::THREADS, PairCfg<R, NL, RL, COLS>::MINB)
 k_last2(Dims d, Symbol<R> Sy, cplx<R>* __restrict__ w, const cplx<R>* __restrict__ tw, int early)
 {
@@ -668,6 +684,14 @@ k_last2(Dims d, Symbol<R> Sy, cplx<R>* __restrict__ w, const cplx<R>* __restrict
     if (sizeof(R) == 4 && early) grid_trigger();  // (a branch, not the predicated form: 137 against 151 us at 256^3)
     col_load<NL, RL, 0>(v[0], a, st);
     col_load<NL, RL, 0>(v[1], b, st);
+    CT* ux = w + ci + (long long)t * ncol;
+    if constexpr (MERGE_X) {
+        CT u[RL];
+        col_load<NL, RL, 0>(u, ux, st);
+        const CT tx = __ldg(Sy.tm[0] + ci);
+#pragma unroll
+        for (int s = 0; s < RL; ++s) v[0][s] = cfma(u[s], tx, v[0][s]);
+    }
     R k2c = Sy.c3.x;
     if (d.D == 3) k2c += __ldg(Sy.k2[0] + ci % d.n0) + __ldg(Sy.k2[1] + ci / d.n0);
     else k2c += __ldg(Sy.k2[0] + ci);
@@ -694,6 +718,12 @@ k_last2(Dims d, Symbol<R> Sy, cplx<R>* __restrict__ w, const cplx<R>* __restrict
     if (valid) {
         col_store<NL, RL, np>(a, st, v[0]);
         col_store<NL, RL, np>(b, st, v[1]);
+        if constexpr (MERGE_X) {
+            const CT tx = __ldg(Sy.td[0] + ci);
+#pragma unroll
+            for (int s = 0; s < RL; ++s) v[1][s] = cmul(v[0][s], tx);
+            col_store<NL, RL, np>(ux, st, v[1]);
+        }
     }
 }
 
@@ -749,9 +779,9 @@ k_deriv2(Dims d, LOp<R> L, const cplx<R>* __restrict__ x, cplx<R>* __restrict__ 
 }
 
 // x axis of the operator and its diagonal: blocks as in k_rows (pair blocks transform p and u_x, the others only
-// combine), w on entry the gradients / divergence of k_deriv2.
+// combine; APART: 2D, one unit a block), w on entry the gradients / divergence of k_deriv2.
 // OP_RESID: w <- y - A_s x, partial (|w|^2, |y|^2);  OP_APPLY: w <- A_s x, no partials.
-template <typename R, int NX, int RX>
+template <typename R, int NX, int RX, bool APART = false>
 __global__ void __launch_bounds__(RowCfg<R, NX, RX>::MAXT, RowCfg<R, NX, RX>::MAXT <= 128 ? 3 : 1)
 k_rows_op(Dims d, Medium<R> M, LOp<R> L, const cplx<R>* __restrict__ x, const cplx<R>* __restrict__ y,
           cplx<R>* __restrict__ w, const cplx<R>* __restrict__ tw, int npair, int nsingle, int mode, int adj,
@@ -763,57 +793,62 @@ k_rows_op(Dims d, Medium<R> M, LOp<R> L, const cplx<R>* __restrict__ x, const cp
     constexpr int np = plan_npass(NX, RX);
     extern __shared__ __align__(128) unsigned char smraw[];
     CT* ex = reinterpret_cast<CT*>(smraw);  // U * SL
-    const int U = blockDim.x / T, H = U >> 1;
-    const int lu = threadIdx.x / T, t = threadIdx.x % T;
+    const int U = APART ? 1 : blockDim.x / T, H = U >> 1;
+    const int lu = APART ? 0 : threadIdx.x / T, t = APART ? threadIdx.x : threadIdx.x % T;
     const long long rpc = d.N / NX;
-    const bool pair = (int)blockIdx.x < npair;
+    const bool pair = !APART && (int)blockIdx.x < npair;
     const int per = pair ? H : U;
     int c, b = blockIdx.x;
     if (pair) {
         c = d.D;
     } else {
         b -= npair;
-        c = 1 + b / nsingle;
+        c = (APART ? 0 : 1) + b / nsingle;
         b = b % nsingle;
     }
     const long long row0 = (long long)b * per;
     const int nrow = (int)(rpc - row0 < per ? rpc - row0 : per);
-    const bool isx = pair && lu >= H;
+    bool isx = pair && lu >= H;
     const int lrow = isx ? lu - H : lu;
     if (isx) c = 0;
     const bool valid = lrow < nrow;
-    const bool pres = pair && !isx;
+    const bool pres = APART ? c == d.D : pair && !isx;
+    if (APART) isx = c == 0;
+    const bool xd = pair || (APART && c != 1);  // an x derivative goes into this unit's row
     const long long rest = row0 + (valid ? lrow : 0);
     const int i1 = (int)(rest % d.n1), i2 = (int)(rest / d.n1);
     const long long vbase = rest * NX;
     const long long fbase = (long long)c * d.N + vbase;
+    const long long fother = (pres ? 0 : (long long)d.D * d.N) + vbase;  // APART: the row whose x derivative comes here
     const RowB<R> rb = row_B(M, d.D, c, i1, i2, vbase);
     CT v[RX];
     grid_wait();
     grid_trigger_if<R>(gridDim.x <= kSMs);
-    if (pair) {
+    if (xd) {
         TwCache<NX, RX, CT> tc;
         tw_load<NX, RX, T>(tc, t, tw);
 #pragma unroll
-        for (int s = 0; s < RX; ++s) v[s] = x[fbase + t + T * slot_q<NX, RX, 0>(s)];
+        for (int s = 0; s < RX; ++s) v[s] = x[(APART ? fother : fbase) + t + T * slot_q<NX, RX, 0>(s)];
         CT* row = ex + (size_t)lu * SL;
         fft_run<NX, RX, -1, true>(v, row, 1, t, tw, tc, RowSync<T>());
 #pragma unroll
         for (int s = 0; s < RX; ++s) {
             CT f = __ldg(L.it[0] + t + T * slot_q<NX, RX, np>(s));  // i g t
-            if (isx) f.x = -f.x;
+            if (APART ? pres : isx) f.x = -f.x;
             v[s] = cmul(v[s], f);
         }
         permute_slots<NX, RX, np, 0>(v);
         fft_run<NX, RX, +1, true>(v, row, 1, t, tw, tc, RowSync<T>());
-        // the pressure's gradient goes to u_x and u_x's divergence to the pressure
-        __syncthreads();
+        // the pressure's gradient goes to u_x and u_x's divergence to the pressure (APART: transformed from the other's row)
+        if constexpr (!APART) {
+            __syncthreads();
 #pragma unroll
-        for (int s = 0; s < RX; ++s) row[s * T + t] = v[s];
-        __syncthreads();
-        const CT* o = ex + (size_t)(isx ? lu - H : lu + H) * SL + t;
+            for (int s = 0; s < RX; ++s) row[s * T + t] = v[s];
+            __syncthreads();
+            const CT* o = ex + (size_t)(isx ? lu - H : lu + H) * SL + t;
 #pragma unroll
-        for (int s = 0; s < RX; ++s) v[s] = o[s * T];
+            for (int s = 0; s < RX; ++s) v[s] = o[s * T];
+        }
     }
     R s0 = (R)0, s1 = (R)0;
     if (valid) {
@@ -833,7 +868,7 @@ k_rows_op(Dims d, Medium<R> M, LOp<R> L, const cplx<R>* __restrict__ x, const cp
             if (adj) dg.y = -dg.y;
             CT a = mk<CT, R>((R)0, (R)0);
             if (!isx) a = w[fbase + i0];
-            if (pair) a = cadd(a, v[s]);
+            if (xd) a = cadd(a, v[s]);
             a = cfma(dg, xv, a);
             if (mode == OP_RESID) {
                 const CT yv = y[fbase + i0];

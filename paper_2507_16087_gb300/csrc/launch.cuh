@@ -101,6 +101,8 @@ cudaError_t launch(Kern kern, long long grid, int threads, size_t smem, cudaStre
 template <typename R> constexpr bool kDependent = sizeof(R) == 4;
 
 constexpr int kWaveBlocks = 2 * kSMs;  // two blocks on every SM
+constexpr int kApartN = 2048;          // row length of rows_apart
+constexpr int kApartRows = 48;         // and the largest extent of its other axis (three blocks a row, an SM each)
 
 // float64 grids whose threads, each with r values, make fewer warps than there are SM sub-partitions (4 an SM)
 template <typename R> inline bool few_warps(long long values, int r)
@@ -187,9 +189,17 @@ template <typename R> inline int early_last(const Dims& d, long long blocks)
 }
 template <typename R> inline int early_rows(const Dims& d, long long blocks) { return early_next<R>(d, blocks, true, 0, 0); }
 
+// 2D grids of few long rows: a block, and so an SM, for every row of a component in place of one for a row of the pressure and
+// of u_x together, whose FP64 instructions (float64) or chain of waits (float32) is the time.  us an iteration, pairs / apart
+// (with every component transformed by itself, as before the scalar form, in brackets): float64 8 x 2048 126 / 68 [79], 48 x
+// 2048 143 / 86 [107]; float32 8 x 2048 10.4 / 7.8 [11.2], 48 x 2048 13.5 / 11.5 [12.9].  Where SMs are short the pairs are
+// better: they save u_x's transforms along y (64 x 2048 144 [175]).
+template <typename R> inline bool rows_apart(const Dims& d) { return d.D == 2 && d.n0 == kApartN && (d.D + 1) * d.n1 <= kSMs; }
+
 // blocks of the row kernels (= norm partials of one iteration)
 template <typename R> inline int rows_blocks(const Plan<R>& P)
 {
+    if (rows_apart<R>(P.d)) return (P.d.D + 1) * P.d.n1;
     switch (P.d.n0) {
 #define CBS_CASE(n) case n: return row_grid<R, n>(P.d).blocks;
         CBS_FOR_EACH_SIZE(CBS_CASE)
@@ -224,17 +234,40 @@ cudaError_t rows_nm(const Plan<R>& P, cplx<R>* x, const cplx<R>* y, cplx<R>* w, 
                   P.d.D == 3 ? early_axis<R>(P.d, g.blocks) : early_last<R>(P.d, g.blocks), adj, nu, partials, P.err);
 }
 
+template <typename R, int N, int RX, int MODE>
+cudaError_t rows_apart_nm(const Plan<R>& P, cplx<R>* x, const cplx<R>* y, cplx<R>* w, int adj, R nu, double* partials,
+                          cudaStream_t st)
+{
+    using Cfg = RowCfg<R, N, RX>;
+    auto kern = k_rows<R, N, RX, MODE, true>;
+    static const cudaError_t attr = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)Cfg::smem_apart(MODE));
+    if (attr != cudaSuccess) return attr;
+    const int blocks = (P.d.D + 1) * P.d.n1;
+    return launch(kern, blocks, Cfg::T, Cfg::smem_apart(MODE), st, kDependent<R> && MODE != ROWS_FWD && MODE != ROWS_COPY, P.d, P.M,
+                  P.Sy[adj ? 1 : 0], x, y, w, P.tw[0], 0, P.d.n1, 1, early_last<R>(P.d, blocks), adj, nu, partials, P.err);
+}
+
+template <typename R, int N, int RX, int MODE>
+cudaError_t rows_any_nm(const Plan<R>& P, cplx<R>* x, const cplx<R>* y, cplx<R>* w, int adj, R nu, double* partials,
+                        cudaStream_t st)
+{
+    if constexpr (N == kApartN) {
+        if (rows_apart<R>(P.d)) return rows_apart_nm<R, N, RX, MODE>(P, x, y, w, adj, nu, partials, st);
+    }
+    return rows_nm<R, N, RX, MODE>(P, x, y, w, adj, nu, partials, st);
+}
+
 template <typename R, int N, int RX>
 cudaError_t rows_rx(const Plan<R>& P, cplx<R>* x, const cplx<R>* y, cplx<R>* w, int mode, int adj, R nu,
                     double* partials, cudaStream_t st)
 {
     switch (mode) {
-    case ROWS_FWD: return rows_nm<R, N, RX, ROWS_FWD>(P, x, y, w, adj, nu, partials, st);
-    case ROWS_FUSED: return rows_nm<R, N, RX, ROWS_FUSED>(P, x, y, w, adj, nu, partials, st);
-    case ROWS_FUSED_NORM: return rows_nm<R, N, RX, ROWS_FUSED_NORM>(P, x, y, w, adj, nu, partials, st);
-    case ROWS_INV: return rows_nm<R, N, RX, ROWS_INV>(P, x, y, w, adj, nu, partials, st);
-    case ROWS_COPY: return rows_nm<R, N, RX, ROWS_COPY>(P, x, y, w, adj, nu, partials, st);
-    case ROWS_GREEN: return rows_nm<R, N, RX, ROWS_GREEN>(P, x, y, w, adj, nu, partials, st);
+    case ROWS_FWD: return rows_any_nm<R, N, RX, ROWS_FWD>(P, x, y, w, adj, nu, partials, st);
+    case ROWS_FUSED: return rows_any_nm<R, N, RX, ROWS_FUSED>(P, x, y, w, adj, nu, partials, st);
+    case ROWS_FUSED_NORM: return rows_any_nm<R, N, RX, ROWS_FUSED_NORM>(P, x, y, w, adj, nu, partials, st);
+    case ROWS_INV: return rows_any_nm<R, N, RX, ROWS_INV>(P, x, y, w, adj, nu, partials, st);
+    case ROWS_COPY: return rows_any_nm<R, N, RX, ROWS_COPY>(P, x, y, w, adj, nu, partials, st);
+    case ROWS_GREEN: return rows_any_nm<R, N, RX, ROWS_GREEN>(P, x, y, w, adj, nu, partials, st);
     default: return cudaErrorInvalidValue;
     }
 }
@@ -267,6 +300,16 @@ cudaError_t rows_op_rx(const Plan<R>& P, const cplx<R>* x, const cplx<R>* y, cpl
                        double* partials, cudaStream_t st)
 {
     using Cfg = RowCfg<R, N, RX>;
+    if constexpr (N == kApartN) {
+        if (rows_apart<R>(P.d)) {
+            auto kern = k_rows_op<R, N, RX, true>;
+            constexpr size_t smem = Cfg::SL * sizeof(cplx<R>);
+            static const cudaError_t attr = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+            if (attr != cudaSuccess) return attr;
+            return launch(kern, (P.d.D + 1) * P.d.n1, Cfg::T, smem, st, kDependent<R>, P.d, P.M, P.L[adj ? 1 : 0], x, y, w, P.tw[0],
+                          0, P.d.n1, mode, adj, partials);
+        }
+    }
     auto kern = k_rows_op<R, N, RX>;
     constexpr int kMax = (int)((size_t)Cfg::UMAX * Cfg::SL * sizeof(cplx<R>));
     static const cudaError_t attr = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, kMax);
@@ -332,10 +375,11 @@ template <typename R> cudaError_t launch_axis(const Plan<R>& P, cplx<R>* w, int 
     }
 }
 
-template <typename R, int N, int RL, int COLS> cudaError_t last2_tile(const Plan<R>& P, cplx<R>* w, int adj, cudaStream_t st)
+template <typename R, int N, int RL, int COLS, bool MERGE_X = false>
+cudaError_t last2_tile(const Plan<R>& P, cplx<R>* w, int adj, cudaStream_t st)
 {
     using Cfg = PairCfg<R, N, RL, COLS>;
-    auto kern = k_last2<R, N, RL, COLS>;
+    auto kern = k_last2<R, N, RL, COLS, MERGE_X>;
     static const cudaError_t attr = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)Cfg::SMEM);
     if (attr != cudaSuccess) return attr;
     const long long blocks = (last_columns(P.d) + COLS - 1) / COLS;
@@ -345,6 +389,9 @@ template <typename R, int N, int RL, int COLS> cudaError_t last2_tile(const Plan
 template <typename R, int N> cudaError_t last2_n(const Plan<R>& P, cplx<R>* w, int adj, cudaStream_t st)
 {
     constexpr int CB = cols_big<R>(N), CS = cols_small<R>(N);
+    if constexpr (N <= kApartRows) {  // (2048 columns of at most 48 points: the small tile's)
+        if (rows_apart<R>(P.d)) return last2_tile<R, N, r_tile<R>(N), CS, true>(P, w, adj, st);
+    }
     if constexpr (has_small_tile<R>(N)) {
         if (small_tiles<R>(N, last_columns(P.d))) return last2_tile<R, N, r_tile<R>(N), CS>(P, w, adj, st);
     }
