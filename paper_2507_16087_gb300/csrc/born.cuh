@@ -107,21 +107,6 @@ __device__ __forceinline__ RowB<R> row_B(const Medium<R>& M, int D, int c, int i
     return rb;
 }
 
-// B from the row's medium values already in registers (m0 = rs_c or kp, m1 = et)
-template <typename R>
-__device__ __forceinline__ cplx<R> born_B_vals(const Medium<R>& M, bool pres, R g, R m0, R m1, bool adj)
-{
-    R vr, vi;
-    if (!pres) {
-        vr = m0 * g - M.a1r;
-        vi = m0 * M.omega - M.a1i;
-    } else {
-        vr = m0 * (g + m1 * M.omega) - M.a2r;
-        vi = m0 * (M.omega - g * m1) - M.a2i;
-    }
-    return mk<cplx<R>, R>((R)1 - vr, adj ? vi : -vi);
-}
-
 template <typename R>
 __device__ __forceinline__ cplx<R> born_B(const Medium<R>& M, const RowB<R>& rb, int i0, bool adj)
 {

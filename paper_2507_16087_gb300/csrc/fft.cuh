@@ -28,7 +28,7 @@ template <> struct real_of<double2> { using T = double; };
 template <typename CT, typename R> __host__ __device__ __forceinline__ CT mk(R a, R b) { CT c; c.x = a; c.y = b; return c; }
 // float32 pairs: one packed instruction (f32x2) where both parts take the same operation, which is most of an FFT's
 // butterflies (each part is rounded as by the scalar instruction).  The kernels issue in 35-45 % of the cycles, so 10-15 %
-// fewer instructions (row kernel at 128^3 29.1 -> 26.1 M) give 2-4 % at 128^3 to 512^3.
+// fewer instructions (row kernel with 16 values a thread at 128^3 29.1 -> 26.1 M) give 2-4 % at 128^3 to 512^3.
 __host__ __device__ __forceinline__ float2 cadd(float2 a, float2 b)
 {
 #if defined(__CUDA_ARCH__) && __CUDA_ARCH__ >= 1000
@@ -93,11 +93,6 @@ template <int S, typename CT> __host__ __device__ __forceinline__ CT cadd_i(CT a
     return a;
 }
 __host__ __device__ __forceinline__ double2 cscale(double2 a, double s) { return make_double2(a.x * s, a.y * s); }
-__host__ __device__ __forceinline__ float2 cconj(float2 a) { return make_float2(a.x, -a.y); }
-__host__ __device__ __forceinline__ double2 cconj(double2 a) { return make_double2(a.x, -a.y); }
-// multiply by s*i  (s = +1 or -1)
-template <int S> __host__ __device__ __forceinline__ float2 mul_si(float2 a) { return S > 0 ? make_float2(-a.y, a.x) : make_float2(a.y, -a.x); }
-template <int S> __host__ __device__ __forceinline__ double2 mul_si(double2 a) { return S > 0 ? make_double2(-a.y, a.x) : make_double2(a.y, -a.x); }
 __host__ __device__ __forceinline__ float cabs2(float2 a) { return a.x * a.x + a.y * a.y; }
 __host__ __device__ __forceinline__ double cabs2(double2 a) { return a.x * a.x + a.y * a.y; }
 
@@ -315,7 +310,7 @@ __device__ __forceinline__ void tw_load(TwCache<N, R, CT>& tc, int tid, const CT
 }
 
 // twiddle table: tw[m] = exp(-2 pi i m / N), m < N
-template <int N, int R, int T, int P, int S, bool USE_TC = true, typename CT>
+template <int N, int R, int T, int P, int S, typename CT>
 __device__ __forceinline__ void pass_compute(CT (&v)[R], int tid, const CT* __restrict__ tw, const TwCache<N, R, CT>& tc)
 {
     constexpr int r = plan_radix(N, R, P);
@@ -328,7 +323,7 @@ __device__ __forceinline__ void pass_compute(CT (&v)[R], int tid, const CT* __re
 #pragma unroll
             for (int k = 1; k < r; ++k) {
                 CT w;
-                if constexpr (USE_TC && TwPolicy<N, R>::cached) w = tc.w[tw_count_before(N, R, P) + m * (r - 1) + k - 1];
+                if constexpr (TwPolicy<N, R>::cached) w = tc.w[tw_count_before(N, R, P) + m * (r - 1) + k - 1];
                 else w = __ldg(&tw[jj * k * (N / (NS * r))]);
                 v[m * r + k] = (S < 0) ? cmul(v[m * r + k], w) : cmulc(v[m * r + k], w);
             }
@@ -386,18 +381,17 @@ __device__ __forceinline__ void pass_exchange(CT (&v)[R], CT* sm, int ss, int ti
 
 // Full transform.  On entry v[s] holds position tid + T*slot_q<N,R,0>(s); on
 // exit v[s] holds position tid + T*slot_q<N,R,npass>(s).
-// USE_TC = false reads every twiddle from the table (for kernels with no registers to spare).
-template <int N, int R, int S, bool PAD = false, int P = 0, bool USE_TC = true, typename CT, typename Sync>
+template <int N, int R, int S, bool PAD = false, int P = 0, typename CT, typename Sync>
 __device__ __forceinline__ void fft_run(CT (&v)[R], CT* sm, int ss, int tid, const CT* __restrict__ tw,
                                         const TwCache<N, R, CT>& tc, Sync sync)
 {
     constexpr int T = N / R;
     constexpr int np = plan_npass(N, R);
     static_assert(np > 0, "unsupported FFT size / register split");
-    pass_compute<N, R, T, P, S, USE_TC>(v, tid, tw, tc);
+    pass_compute<N, R, T, P, S>(v, tid, tw, tc);
     if constexpr (P + 1 < np) {
         pass_exchange<N, R, T, P, PAD>(v, sm, ss, tid, sync);
-        fft_run<N, R, S, PAD, P + 1, USE_TC>(v, sm, ss, tid, tw, tc, sync);
+        fft_run<N, R, S, PAD, P + 1>(v, sm, ss, tid, tw, tc, sync);
     }
 }
 

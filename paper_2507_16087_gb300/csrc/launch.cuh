@@ -22,6 +22,7 @@ template <typename R> __host__ __device__ constexpr int r_axis(int n)
 {
     return (n % 3 == 0) ? 12 : ((sizeof(R) == 4 && n >= 128) ? 16 : 8);
 }
+// (the last axis takes the other strided axis's split, whatever the number of components)
 template <typename R> __host__ __device__ constexpr int r_last(int n, int = 2) { return r_axis<R>(n); }
 // small grids: fewer values a thread, so that a transform has more threads.  float32 (see small_tiles): 8 at every 2^k
 // extent.  float64 (see few_warps): 4, and 6 up to 48 points: an SM sub-partition issues one FP64 warp instruction in
@@ -192,8 +193,8 @@ template <typename R> inline int early_rows(const Dims& d, long long blocks) { r
 // 2D grids of few long rows: a block, and so an SM, for every row of a component in place of one for a row of the pressure and
 // of u_x together, whose FP64 instructions (float64) or chain of waits (float32) is the time.  us an iteration, pairs / apart
 // (with every component transformed by itself, as before the scalar form, in brackets): float64 8 x 2048 126 / 68 [79], 48 x
-// 2048 143 / 86 [107]; float32 8 x 2048 10.4 / 7.8 [11.2], 48 x 2048 13.5 / 11.5 [12.9].  Where SMs are short the pairs are
-// better: they save u_x's transforms along y (64 x 2048 144 [175]).
+// 2048 143 / 86 [107]; float32 8 x 2048 10.4 / 7.8 [11.2], 48 x 2048 13.5 / 11.5 [12.9].  With more rows an SM has two
+// of them either way, and the last axis of the pairs carries no third field (64 x 2048 144 [175]).
 template <typename R> inline bool rows_apart(const Dims& d) { return d.D == 2 && d.n0 == kApartN && (d.D + 1) * d.n1 <= kSMs; }
 
 // blocks of the row kernels (= norm partials of one iteration)
