@@ -1220,9 +1220,10 @@ void set_l2_window(cbs_solver* s, void* base, size_t bytes)
     cudaDeviceGetAttribute(&max_persist, cudaDevAttrMaxPersistingL2CacheSize, dev);
     cudaDeviceGetAttribute(&max_window, cudaDevAttrMaxAccessPolicyWindowSize, dev);
     if (max_persist <= 0 || max_window <= 0) return;
-    // Only a field that fits in the persisting carve-out gets a window.  A window over a larger field
-    // marks most of its accesses streaming (evict first) and measured 1.7-1.9x slower per iteration
-    // on GB300 at 256^3 and 512^3; at 128^3 (67 MB) the window makes an iteration 7 % faster.
+    // Only fields that fit in the persisting carve-out (67.7 MB on GB300) get a window.  A window over
+    // larger ones marks most of their accesses streaming (evict first) and measured 1.7-1.9x slower per
+    // iteration at 256^3 and 512^3.  us an iteration without / with it: 128^3 (50 MB) 100.8 / 94.3, 2048^2
+    // (67.1 MB) 215 / 202, 2048 x 1024 102 / 98, 64^3 and 96^3 the same.
     if (bytes > (size_t)max_persist || bytes > (size_t)max_window) return;
     const size_t win = bytes;
     size_t cur = 0;
