@@ -109,7 +109,7 @@ class Server:
     exclusive_voxels: requests with at least this many voxels (grids whose kernels fill the GPU on their own:
     1024^2, 128^3 and larger by default) run one at a time among themselves; smaller requests are admitted beside
     them and may pass a large request that waits for the running one.  Measured on the 256-request mixed stream
-    at 0.8 x its saturated rate: p50 0.19 s / p99 1.86 s (with slower kernels, 0.33 s / 2.51 s against 0.56 s /
+    at 0.8 x its saturated rate: p50 0.19 s / p99 1.84 s (with slower kernels, 0.33 s / 2.51 s against 0.56 s /
     2.91 s in plain arrival order, with a 3 % higher saturated rate).  None or 0: every request is admitted in arrival order while slots and memory
     last."""
 
